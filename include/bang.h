@@ -59,6 +59,7 @@ typedef struct bang_search_params {
     /* Optional per-query outputs (nq entries each), host or device:
      * expansions (the paper's iteration count I, §7.7), status (0 = converged,
      * 1 = stopped by iter_cap, 2 = its tensor-core table could not be built,
+     * 3 = a bounded wait inside the search gave up,
      * -1 = its k or L out of range in the batched form), and PQ distances
      * computed (§4.4). */
     uint32_t *out_iters;
@@ -73,7 +74,8 @@ typedef struct bang_search_params {
      * distances (§4.4), next-node choice and prefetch (§4.5), re-rank
      * candidate (§4.8), merge remainder, merge ranking of the new keys and
      * merge shifting of the worklist (§4.6-§4.7), and the query's total: the
-     * paper's per-kernel GPU-time breakdown (§7.3) for the fused kernel. */
+     * paper's per-kernel GPU-time breakdown (§7.3) for the fused kernel, taken
+     * in its one-warp form. */
     unsigned long long *out_phase_cycles;
     /* Distance mode (bang_mode): PQ distances from an FP32 table (0, the
      * default, bit-exact with the reference order), from a BF16 table summed
@@ -108,14 +110,17 @@ typedef struct bang_search_params {
     /* How many candidates for the next node are requested per iteration: 0
      * or 1 = the chosen one only, after the distances (§4.5's eager choice);
      * 2 = also the first unvisited worklist entry after u*, at the start of
-     * the iteration (used when it is chosen, wasted otherwise).  Results do
+     * the iteration (used when it is chosen, wasted otherwise).  Only where one
+     * warp searches a query alone; where several do (few queries per SM, or
+     * the FP32 table), the next entries are always expanded ahead.  Results do
      * not depend on it. */
     uint32_t prefetch_depth;
     /* When the new neighbours' PQ code rows are requested: 0 = after the seen
      * filter, only the new ones; 1 = every neighbour's row as soon as the
      * expanded node's row arrives, so that the filter runs while they are in
      * flight (used when R <= 64, d <= 128 and M <= 32, and without
-     * BANG_NEIGHBOR_CODES; otherwise ignored).  Results do not depend on it. */
+     * BANG_NEIGHBOR_CODES, where one warp searches a query alone; otherwise
+     * ignored).  Results do not depend on it. */
     uint32_t early_codes;
     /* How the re-rank of §4.8 runs (modes 0, 1 and 3; mode 2 has none):
      * 0 = fused into the loop (each expanded node's vector arrives with its

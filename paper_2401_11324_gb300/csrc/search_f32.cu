@@ -1,9 +1,9 @@
-// Instantiates the search kernel for one distance mode (see search_kernel.cuh).
-#include "search_kernel.cuh"
+// Instantiates the search kernel for one distance mode (see search_team.cuh).
+#include "search_team.cuh"
 
 namespace bang {
 cudaError_t launch_search_f32(const SearchArgs &a, int dtype, size_t smem, cudaStream_t st)
 {
-    return launch_mode<kModeF32>(a, dtype, smem, st);
+    return launch_team<kModeF32>(a, dtype, smem, st);
 }
 }  // namespace bang

@@ -332,6 +332,29 @@ def test_phase_clock_instantiation_gives_identical_results(u8small, mode, flags)
 
 
 @pytest.mark.parametrize("mode", [0, 1, 2, 3])
+@pytest.mark.parametrize("nq", [1, 400, 1300, 3000])
+def test_team_form_equals_the_one_warp_form(u8small, cfg1, mode, nq):
+    # a query is searched by one warp or by a control warp with two or three
+    # expanders, chosen by how many queries share an SM; the phase clock always
+    # runs the one-warp form.  Everything is equal, to the last bit: one- and
+    # two-word filter positions, top-k in registers and in shared memory, the
+    # smallest worklists, and caps that end a search between two expansions.
+    for w in (u8small, cfg1):
+        Q = np.resize(w["queries"], (nq, w["queries"].shape[1]))
+        for k, L, log2z, cap, rerank in ((10, 64, 16, 0, 0), (1, 1, 10, 0, 0), (40, 70, 17, 0, 0),
+                                         (10, 32, 14, 7, 0), (10, 48, 16, 8, 2), (5, 130, 16, 0, 1)):
+            if mode == 2 and rerank:
+                rerank = 0
+            kw = dict(log2z=log2z, iter_cap=cap, trace_cap=400, mode=mode, rerank=rerank)
+            ref = gpu_search(w, Q, k, L, phases=True, **kw)
+            g = gpu_search(w, Q, k, L, **kw)
+            for f in ("ids", "dist", "iters", "ndist", "status"):
+                assert (g[f] == ref[f]).all(), (mode, nq, k, L, log2z, cap, rerank, f)
+            seen = np.arange(400)[None] < ref["iters"][:, None]
+            assert (g["trace"][seen] == ref["trace"][seen]).all()
+
+
+@pytest.mark.parametrize("mode", [0, 1, 2, 3])
 def test_node_records_give_identical_results(u8small, cfg1, mode):
     # BANG_NODE_RECORDS: each node's row and vector in one host record
     R, P, N = bang.BANG_NODE_RECORDS, bang.BANG_GRAPH_PACKED, bang.BANG_NEIGHBOR_CODES
