@@ -5,14 +5,21 @@
 // (no fused multiply-add); ties go to the smaller id.  The only FP64 on the
 // GPU in this library besides the offline k-means.
 //
-// Three passes.  (1) Each query's exact k nearest among the first S points
-// (S = min(n, 262144)) give a threshold: the k-th of them is at least the
-// k-th over all n points, so every true neighbour is within it.  (2) A tile
-// of queries held in shared memory streams over all points, one point per
-// thread, and appends every point within a query's threshold to that query's
-// candidate list.  (3) One warp per query picks the k smallest candidates by
-// (distance, id).  A list that overflows its capacity is detected and pass 2
-// rerun with room for the longest list.
+// The k-th distance among any subset of the points is at least the k-th over
+// all n, so every true neighbour lies within it.  (1) Each query's exact k
+// nearest among 4,096 points (spread evenly over the ids) give a first
+// threshold.  (2) A tile of queries held in shared memory streams over 16
+// times as many points, one point per thread, and appends every point within a
+// query's threshold to that query's candidate list (about 16 k of them); their
+// k-th distance is the next threshold, and so on until all n points have been
+// streamed over.  (3) One warp per query picks the k smallest candidates of
+// the last list by (distance, id).  A list that overflows its capacity is
+// detected and its pass rerun with room for the longest list.
+//
+// Step (1) keeps each query's k nearest sorted in one warp, a serial chain per
+// insertion: over 262,144 points it took 294 of 375 ms (10,000 u8 queries,
+// d = 128, 1M points, k = 100); over 4,096, 6 of 84 ms, the level added in
+// between included.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -30,12 +37,14 @@ constexpr uint32_t kNo = 0xFFFFFFFFu;
 constexpr int kW = 32;
 constexpr int kKPL = 8;                  // top-k entries per lane in pass 1: k <= 256
 constexpr uint32_t kTileQ = 128;         // at most this many queries per CTA in pass 2
-constexpr uint32_t kSample = 262144;
+constexpr uint32_t kSample = 4096;       // points of the first threshold
+constexpr uint32_t kLevel = 16;          // each further level streams over this many times as many
 
 struct GtArgs {
     const void *base, *queries;
     int dtype;
-    uint64_t n;
+    uint64_t n;                  // points of this level: ids i * stride, i < n
+    uint64_t stride;
     uint32_t nq, d, k;
     const double *thr;           // nq thresholds (pass 2)
     double *thr_out;             // pass 1
@@ -110,10 +119,11 @@ __device__ __forceinline__ bool less_pair(uint64_t da, uint32_t ia, uint64_t db,
     return da < db || (da == db && ia < ib);
 }
 
-// Pass 1: one warp per query, the exact k nearest of the first S points kept
+// Step 1: one warp per query, the exact k nearest of the level's points kept
 // sorted across the warp (8 per lane); the threshold is the k-th distance.
-__global__ void sample_threshold(const GtArgs g, uint64_t S)
+__global__ void sample_threshold(const GtArgs g)
 {
+    const uint64_t S = g.n;
     const int lane = threadIdx.x & 31;
     const uint32_t q = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     if (q >= g.nq) return;
@@ -130,7 +140,7 @@ __global__ void sample_threshold(const GtArgs g, uint64_t S)
         uint64_t dk = ~0ull;
         uint32_t ik = kNo;
         if (i < S) {
-            dk = static_cast<uint64_t>(__double_as_longlong(dist_rows(g, qr, i)));
+            dk = static_cast<uint64_t>(__double_as_longlong(dist_rows(g, qr, i * g.stride)));
             ik = static_cast<uint32_t>(i);
         }
         uint32_t want = __ballot_sync(0xFFFFFFFFu, ik != kNo && less_pair(dk, ik, thd, thi));
@@ -171,7 +181,7 @@ __global__ void sample_threshold(const GtArgs g, uint64_t S)
                                   : __longlong_as_double(0x7FF0000000000000ll);
 }
 
-// Pass 2: blockIdx.y = tile of kTileQ queries (rows in shared memory);
+// Step 2: blockIdx.y = tile of kTileQ queries (rows in shared memory);
 // threads stride over the points.
 __global__ void collect(const GtArgs g)
 {
@@ -184,8 +194,9 @@ __global__ void collect(const GtArgs g)
     __shared__ double th[kTileQ];
     if (threadIdx.x < nt) th[threadIdx.x] = g.thr[q0 + threadIdx.x];
     __syncthreads();
-    for (uint64_t i = blockIdx.x * static_cast<uint64_t>(blockDim.x) + threadIdx.x; i < g.n;
-         i += static_cast<uint64_t>(gridDim.x) * blockDim.x) {
+    for (uint64_t i0 = blockIdx.x * static_cast<uint64_t>(blockDim.x) + threadIdx.x; i0 < g.n;
+         i0 += static_cast<uint64_t>(gridDim.x) * blockDim.x) {
+        const uint64_t i = i0 * g.stride;
         uint4 xr[8];                     // the point's row, for the register path
         const uint32_t nv = g.d / 16u;
         if (g.regrow) {
@@ -225,7 +236,66 @@ __global__ void collect(const GtArgs g)
     }
 }
 
-// Pass 3: one warp per query, the k smallest candidates in (distance, id) order.
+// The threshold of the next level: an upper bound of the k-th smallest distance
+// of a query's list (its FP32 value rounded up; integer distances are exact),
+// by four rounds of 8-bit digits.  One warp per query.
+constexpr int kKthWarps = 4;
+__global__ void __launch_bounds__(kKthWarps * kW) kth_threshold(const GtArgs g)
+{
+    __shared__ uint32_t hist[kKthWarps][256];
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    const uint32_t q = blockIdx.x * kKthWarps + wid;
+    if (q >= g.nq) return;
+    const uint32_t m = g.cnt[q];                 // at most cap, checked by the host
+    const double *cd = g.cd + static_cast<uint64_t>(q) * g.cap;
+    if (m < g.k) {                               // fewer than k points so far: no threshold
+        if (lane == 0) g.thr_out[q] = __longlong_as_double(0x7FF0000000000000ll);
+        return;
+    }
+    uint32_t prefix = 0, mask = 0, want = g.k;   // the want-th among the values with this prefix
+    for (int shift = 24; shift >= 0; shift -= 8) {
+        for (int b = lane; b < 256; b += kW) hist[wid][b] = 0;
+        __syncwarp();
+        for (uint32_t j = lane; j < m; j += kW) {
+            const uint32_t v = __float_as_uint(__double2float_ru(cd[j]));
+            if ((v & mask) == prefix) atomicAdd(&hist[wid][(v >> shift) & 255u], 1u);
+        }
+        __syncwarp();
+        uint32_t h[8], sum = 0;                  // this lane's bins: 8 lane .. 8 lane + 7
+#pragma unroll
+        for (int b = 0; b < 8; ++b) {
+            h[b] = hist[wid][lane * 8 + b];
+            sum += h[b];
+        }
+        uint32_t below = sum;
+#pragma unroll
+        for (int o = 1; o < kW; o <<= 1) {
+            const uint32_t up = __shfl_up_sync(0xFFFFFFFFu, below, o);
+            if (lane >= o) below += up;
+        }
+        below -= sum;
+        const bool here = below < want && want <= below + sum;
+        uint32_t bin = 0, left = here ? want - below : 0u;
+        if (here) {
+#pragma unroll
+            for (int b = 0; b < 7; ++b)
+                if (bin == static_cast<uint32_t>(b) && left > h[b]) {
+                    left -= h[b];
+                    ++bin;
+                }
+            bin += lane * 8u;
+        }
+        const int src = __ffs(__ballot_sync(0xFFFFFFFFu, here)) - 1;
+        bin = __shfl_sync(0xFFFFFFFFu, bin, src);
+        want = __shfl_sync(0xFFFFFFFFu, left, src);
+        prefix |= bin << shift;
+        mask |= 255u << shift;
+        __syncwarp();
+    }
+    if (lane == 0) g.thr_out[q] = static_cast<double>(__uint_as_float(prefix));
+}
+
+// Step 3: one warp per query, the k smallest candidates in (distance, id) order.
 __global__ void select_k(const GtArgs g)
 {
     const int lane = threadIdx.x & 31;
@@ -340,7 +410,6 @@ extern "C" int bang_ground_truth(int device, const void *base, const void *queri
         GT_TRY(cudaMemcpyAsync(dq.p, queries, static_cast<uint64_t>(nq) * d * esz, cudaMemcpyHostToDevice, st));
         Q = dq.p;
     }
-    const uint64_t S = n < kSample ? n : kSample;
     DArr<double> thr, cd, odist;
     DArr<uint32_t> cnt, ci, oids;
     GT_TRY(thr.alloc(nq));
@@ -350,7 +419,6 @@ extern "C" int bang_ground_truth(int device, const void *base, const void *queri
     g.base = B;
     g.queries = Q;
     g.dtype = dtype;
-    g.n = n;
     g.nq = nq;
     g.d = d;
     g.k = k;
@@ -363,31 +431,42 @@ extern "C" int bang_ground_truth(int device, const void *base, const void *queri
         g.words = dtype != BANG_F32 && d % 4 == 0 && ab % 4 == 0 && aq % 4 == 0;
         g.regrow = dtype != BANG_F32 && d % 16 == 0 && d <= 128 && ab % 16 == 0;
     }
-    sample_threshold<<<(nq + 3) / 4, 128, 0, st>>>(g, S);
+    g.n = n < kSample ? n : kSample;
+    g.stride = n / g.n;
+    sample_threshold<<<(nq + 3) / 4, 128, 0, st>>>(g);
     GT_TRY(cudaGetLastError());
-    // expected list length about k * n / S; room for twice that, then the longest
-    uint64_t cap = 2ull * k * ((n + S - 1) / S) + 256;
     int sms = 0;
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, device);
     const uint32_t tiles = (nq + tileq - 1) / tileq;
     const uint32_t gx = static_cast<uint32_t>((static_cast<uint64_t>(sms) * 8 + tiles - 1) / tiles) + 1;
-    for (int attempt = 0; attempt < 2; ++attempt) {
-        GT_TRY(cd.alloc(cap * nq));
-        GT_TRY(ci.alloc(cap * nq));
-        GT_TRY(cudaMemsetAsync(cnt.p, 0, nq * 4, st));
-        g.cd = cd.p;
-        g.ci = ci.p;
-        g.cap = cap;
-        collect<<<dim3(gx, tiles), 256, tileq * d * esz, st>>>(g);
+    std::vector<uint32_t> c(nq);
+    uint64_t cap = 0;
+    for (uint64_t seen = g.n;; seen = g.n) {
+        g.n = seen < n / kLevel ? seen * kLevel : n;     // the last level takes every point
+        g.stride = n / g.n;
+        // expected list length about k * (points now / points before); room for twice that, then the longest
+        uint64_t room = 2ull * k * ((g.n + seen - 1) / seen) + 256;
+        for (int attempt = 0;; ++attempt) {
+            if (room > cap) {
+                GT_TRY(cd.alloc(room * nq));
+                GT_TRY(ci.alloc(room * nq));
+                cap = room;
+            }
+            GT_TRY(cudaMemsetAsync(cnt.p, 0, nq * 4, st));
+            g.cd = cd.p;
+            g.ci = ci.p;
+            g.cap = cap;
+            collect<<<dim3(gx, tiles), 256, tileq * d * esz, st>>>(g);
+            GT_TRY(cudaGetLastError());
+            GT_TRY(cudaMemcpyAsync(c.data(), cnt.p, nq * 4, cudaMemcpyDeviceToHost, st));
+            GT_TRY(cudaStreamSynchronize(st));
+            room = *std::max_element(c.begin(), c.end());
+            if (room <= cap) break;
+            if (attempt == 1) return gtfail(BANG_ECUDA, "bang_ground_truth: candidate lists kept growing");
+        }
+        if (g.n == n) break;
+        kth_threshold<<<(nq + kKthWarps - 1) / kKthWarps, kKthWarps * kW, 0, st>>>(g);
         GT_TRY(cudaGetLastError());
-        std::vector<uint32_t> c(nq);
-        GT_TRY(cudaMemcpyAsync(c.data(), cnt.p, nq * 4, cudaMemcpyDeviceToHost, st));
-        GT_TRY(cudaStreamSynchronize(st));
-        uint64_t mx = 0;
-        for (uint32_t i = 0; i < nq; ++i) mx = c[i] > mx ? c[i] : mx;
-        if (mx <= cap) break;
-        if (attempt == 1) return gtfail(BANG_ECUDA, "bang_ground_truth: candidate lists kept growing");
-        cap = mx;
     }
     const bool dev_out = is_dev(out_ids);
     if (!dev_out) {

@@ -140,3 +140,19 @@ def test_ground_truth_bit_exact(dt, n, d, k, nq):
     assert (ids == ids_o).all(), np.argwhere(ids != ids_o)[:5]
     fin = np.isfinite(dist_o)
     assert (np.isfinite(dist) == fin).all() and (dist[fin] == dist_o[fin]).all()
+
+
+@pytest.mark.parametrize("dt,d", [("u8", 16), ("i8", 33), ("f32", 8)])
+@pytest.mark.parametrize("n,k", [(4095, 256), (4097, 1), (65_536, 100), (65_537, 3), (140_000, 17)])
+def test_ground_truth_levels(dt, d, n, k):
+    # around the sizes where a level of thresholds comes in, with the rows
+    # sorted (neighbours share ids), with many equal distances, and a query
+    # that is a point
+    rng = np.random.default_rng(n + k)
+    X = rng.integers(0, 12, size=(n, d))
+    X = X[np.lexsort(X.T[::-1])]
+    X = X.astype({"u8": np.uint8, "i8": np.int8, "f32": np.float32}[dt])
+    Q = np.ascontiguousarray(X[rng.choice(n, 9)])
+    ref_ids, ref_dist = oracle.bruteforce_knn(X, Q, k)
+    ids, dist = bang.bang_ground_truth(X, Q, k)
+    assert (ids == ref_ids).all() and (dist == ref_dist).all()
