@@ -156,3 +156,33 @@ def test_ground_truth_levels(dt, d, n, k):
     ref_ids, ref_dist = oracle.bruteforce_knn(X, Q, k)
     ids, dist = bang.bang_ground_truth(X, Q, k)
     assert (ids == ref_ids).all() and (dist == ref_dist).all()
+
+
+@pytest.mark.parametrize("dt,d,M,ns,what", [
+    ("u8", 5, 5, 1001, "few values"),      # 1-wide subspaces, distance ties everywhere
+    ("u8", 34, 16, 2999, "few values"),    # 3- and 2-wide
+    ("i8", 32, 2, 513, "any"),             # 16-wide, the widest
+    ("i8", 21, 4, 2, "any"),               # 6- and 5-wide, two training points
+    ("f32", 9, 2, 1003, "any"),            # 5- and 4-wide
+    ("f32", 8, 2, 1000, "huge"),           # FP32 distances overflow
+    ("f32", 8, 2, 1000, "tiny"),           # FP32 products underflow
+    ("f32", 12, 3, 1000, "close"),         # distances that FP32 cannot tell apart
+])
+def test_pq_build_where_fp32_is_not_enough(dt, d, M, ns, what):
+    rng = np.random.default_rng(d * 11 + M)
+    n = 3000
+    if dt == "f32":
+        X = rng.normal(size=(n, d))
+        X = X * {"any": 3.0, "huge": 1e25, "tiny": 1e-24, "close": 1e-7}[what]
+        X = (X + 1.0 if what == "close" else X).astype(np.float32)
+    elif what == "few values":
+        X = rng.integers(0, 5, size=(n, d)).astype(np.uint8)
+    else:
+        X = rng.integers(-128, 128, size=(n, d)).astype(np.int8)
+    sample = np.sort(rng.choice(n, size=ns, replace=False)).astype(np.uint64)
+    init = np.stack([rng.choice(n, size=256, replace=False) for _ in range(M)]).astype(np.uint64)
+    cb_ref = oracle.pq_train(X.astype(np.float32), M, sample, init, 3)
+    codes_ref = oracle.pq_encode(X, M, cb_ref)
+    cb, codes = bang.bang_build_pq(X, M, sample, init, 3)
+    assert (cb.view(np.uint32) == cb_ref.view(np.uint32)).all()
+    assert (codes == codes_ref).all()
