@@ -7,19 +7,22 @@
 //
 // The k-th distance among any subset of the points is at least the k-th over
 // all n, so every true neighbour lies within it.  (1) Each query's exact k
-// nearest among 4,096 points (spread evenly over the ids) give a first
+// nearest among 1,024 points (spread evenly over the ids) give a first
 // threshold.  (2) A tile of queries held in shared memory streams over 16
 // times as many points, one point per thread, and appends every point within a
 // query's threshold to that query's candidate list (about 16 k of them); their
 // k-th distance is the next threshold, and so on until all n points have been
-// streamed over.  (3) One warp per query picks the k smallest candidates of
+// streamed over; integer rows of up to 256 dimensions and FP32 rows of up to
+// 128 on the tensor cores (ground_truth_tc.cuh), others as above.  (3) One warp per query picks the k smallest candidates of
 // the last list by (distance, id).  A list that overflows its capacity is
 // detected and its pass rerun with room for the longest list.
 //
 // Step (1) keeps each query's k nearest sorted in one warp, a serial chain per
 // insertion: over 262,144 points it took 294 of 375 ms (10,000 u8 queries,
-// d = 128, 1M points, k = 100); over 4,096, 6 of 84 ms, the level added in
-// between included.
+// d = 128, 1M points, k = 100), over 1,024 it takes 2.2.  The streamed levels
+// are a contraction: with a point per thread (vabsdiff4 + dp4a) they took 73
+// ms, on the tensor cores 7.6; the sorted selection took 3.9 ms one neighbour
+// after the other, 0.1 gathered and sorted.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -30,6 +33,7 @@
 
 #include "bang.h"
 #include "bang_internal.h"
+#include "ground_truth_tc.cuh"
 
 namespace {
 
@@ -37,7 +41,7 @@ constexpr uint32_t kNo = 0xFFFFFFFFu;
 constexpr int kW = 32;
 constexpr int kKPL = 8;                  // top-k entries per lane in pass 1: k <= 256
 constexpr uint32_t kTileQ = 128;         // at most this many queries per CTA in pass 2
-constexpr uint32_t kSample = 4096;       // points of the first threshold
+constexpr uint32_t kSample = 1024;       // points of the first threshold
 constexpr uint32_t kLevel = 16;          // each further level streams over this many times as many
 
 struct GtArgs {
@@ -236,35 +240,26 @@ __global__ void collect(const GtArgs g)
     }
 }
 
-// The threshold of the next level: an upper bound of the k-th smallest distance
-// of a query's list (its FP32 value rounded up; integer distances are exact),
-// by four rounds of 8-bit digits.  One warp per query.
-constexpr int kKthWarps = 4;
-__global__ void __launch_bounds__(kKthWarps * kW) kth_threshold(const GtArgs g)
+// An upper bound of the k-th smallest of m >= k distances, as FP32 bits: its
+// FP32 value rounded up (integer distances are exact), by four rounds of 8-bit
+// digits.  One warp; hist: 256 words of shared memory.
+__device__ __forceinline__ uint32_t value_bits(double d) { return __float_as_uint(__double2float_ru(d)); }
+
+__device__ __forceinline__ uint32_t kth_bits(const double *cd, uint32_t m, uint32_t k, uint32_t *hist, int lane)
 {
-    __shared__ uint32_t hist[kKthWarps][256];
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    const uint32_t q = blockIdx.x * kKthWarps + wid;
-    if (q >= g.nq) return;
-    const uint32_t m = g.cnt[q];                 // at most cap, checked by the host
-    const double *cd = g.cd + static_cast<uint64_t>(q) * g.cap;
-    if (m < g.k) {                               // fewer than k points so far: no threshold
-        if (lane == 0) g.thr_out[q] = __longlong_as_double(0x7FF0000000000000ll);
-        return;
-    }
-    uint32_t prefix = 0, mask = 0, want = g.k;   // the want-th among the values with this prefix
+    uint32_t prefix = 0, mask = 0, want = k;     // the want-th among the values with this prefix
     for (int shift = 24; shift >= 0; shift -= 8) {
-        for (int b = lane; b < 256; b += kW) hist[wid][b] = 0;
+        for (int b = lane; b < 256; b += kW) hist[b] = 0;
         __syncwarp();
         for (uint32_t j = lane; j < m; j += kW) {
-            const uint32_t v = __float_as_uint(__double2float_ru(cd[j]));
-            if ((v & mask) == prefix) atomicAdd(&hist[wid][(v >> shift) & 255u], 1u);
+            const uint32_t v = value_bits(cd[j]);
+            if ((v & mask) == prefix) atomicAdd(&hist[(v >> shift) & 255u], 1u);
         }
         __syncwarp();
         uint32_t h[8], sum = 0;                  // this lane's bins: 8 lane .. 8 lane + 7
 #pragma unroll
         for (int b = 0; b < 8; ++b) {
-            h[b] = hist[wid][lane * 8 + b];
+            h[b] = hist[lane * 8 + b];
             sum += h[b];
         }
         uint32_t below = sum;
@@ -292,25 +287,93 @@ __global__ void __launch_bounds__(kKthWarps * kW) kth_threshold(const GtArgs g)
         mask |= 255u << shift;
         __syncwarp();
     }
-    if (lane == 0) g.thr_out[q] = static_cast<double>(__uint_as_float(prefix));
+    return prefix;
 }
 
-// Step 3: one warp per query, the k smallest candidates in (distance, id) order.
-__global__ void select_k(const GtArgs g)
+constexpr int kKthWarps = 4;
+
+// The threshold of the next level from a query's list.  One warp per query.
+__global__ void __launch_bounds__(kKthWarps * kW) kth_threshold(const GtArgs g)
 {
-    const int lane = threadIdx.x & 31;
-    const uint32_t q = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    __shared__ uint32_t hist[kKthWarps][256];
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    const uint32_t q = blockIdx.x * kKthWarps + wid;
     if (q >= g.nq) return;
-    const uint64_t m = g.cnt[q] < g.cap ? g.cnt[q] : g.cap;
+    const uint32_t m = g.cnt[q];                 // at most cap, checked by the host
+    double t = __longlong_as_double(0x7FF0000000000000ll);       // fewer than k points so far: no threshold
+    if (m >= g.k)
+        t = static_cast<double>(__uint_as_float(kth_bits(g.cd + static_cast<uint64_t>(q) * g.cap, m, g.k, hist[wid], lane)));
+    if (lane == 0) g.thr_out[q] = t;
+}
+
+// Step 3: one warp per query, the k smallest candidates in (distance, id)
+// order: those within the bound of the k-th (k of them, and what ties with it
+// or rounds to it) are gathered and bitonic-sorted in shared memory; when more
+// than kSortMax are, the k smallest are taken one after the other.
+constexpr uint32_t kSortMax = 512;
+__global__ void __launch_bounds__(kKthWarps * kW) select_k(const GtArgs g)
+{
+    __shared__ uint32_t hist[kKthWarps][256];
+    __shared__ uint64_t sd[kKthWarps][kSortMax];
+    __shared__ uint32_t si[kKthWarps][kSortMax];
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    const uint32_t q = blockIdx.x * kKthWarps + wid;
+    if (q >= g.nq) return;
+    const uint32_t m = static_cast<uint32_t>(g.cnt[q] < g.cap ? g.cnt[q] : g.cap);
     const double *cd = g.cd + static_cast<uint64_t>(q) * g.cap;
     const uint32_t *ci = g.ci + static_cast<uint64_t>(q) * g.cap;
+    const uint32_t bound = m >= g.k ? kth_bits(cd, m, g.k, hist[wid], lane) : 0xFFFFFFFFu;
+    uint32_t c = 0;                              // gathered
+    for (uint32_t j0 = 0; j0 < m && c <= kSortMax; j0 += kW) {
+        const uint32_t j = j0 + lane;
+        const bool in = j < m && value_bits(cd[j]) <= bound;
+        const uint32_t bal = __ballot_sync(0xFFFFFFFFu, in);
+        const uint32_t at = c + __popc(bal & ((1u << lane) - 1u));
+        if (in && at < kSortMax) {
+            sd[wid][at] = static_cast<uint64_t>(__double_as_longlong(cd[j]));
+            si[wid][at] = ci[j];
+        }
+        c += __popc(bal);
+    }
+    if (c <= kSortMax) {
+        uint32_t P = kW;
+        while (P < c) P <<= 1;
+        for (uint32_t i = c + lane; i < P; i += kW) {
+            sd[wid][i] = ~0ull;
+            si[wid][i] = kNo;
+        }
+        __syncwarp();
+        for (uint32_t size = 2; size <= P; size <<= 1)
+            for (uint32_t j = size >> 1; j > 0; j >>= 1) {
+                for (uint32_t t = lane; t < P / 2; t += kW) {
+                    const uint32_t i = ((t & ~(j - 1u)) << 1) | (t & (j - 1u)), l = i | j;
+                    const uint64_t xd = sd[wid][i], yd = sd[wid][l];
+                    const uint32_t xi = si[wid][i], yi = si[wid][l];
+                    const bool up = (i & size) == 0;
+                    if (less_pair(yd, yi, xd, xi) == up) {
+                        sd[wid][i] = yd;
+                        si[wid][i] = yi;
+                        sd[wid][l] = xd;
+                        si[wid][l] = xi;
+                    }
+                }
+                __syncwarp();
+            }
+        for (uint32_t r = lane; r < g.k; r += kW) {
+            const uint64_t o = static_cast<uint64_t>(q) * g.k + r;
+            const bool have = r < c;
+            g.out_ids[o] = have ? si[wid][r] : kNo;
+            g.out_dist[o] = __longlong_as_double(have ? static_cast<long long>(sd[wid][r]) : 0x7FF0000000000000ll);
+        }
+        return;
+    }
     uint64_t pd = 0;             // the last pair taken (exclusive lower bound)
     uint32_t pi = 0;
     bool first = true;
     for (uint32_t r = 0; r < g.k; ++r) {
         uint64_t bd = ~0ull;
         uint32_t bi = kNo;
-        for (uint64_t j = lane; j < m; j += kW) {
+        for (uint32_t j = lane; j < m; j += kW) {
             const uint64_t dj = static_cast<uint64_t>(__double_as_longlong(cd[j]));
             const uint32_t ij = ci[j];
             if (!first && !less_pair(pd, pi, dj, ij)) continue;          // already taken
@@ -341,6 +404,86 @@ template <typename T> struct DArr {
         if (p) cudaFree(p);
         p = nullptr;
         return cudaMalloc(&p, sizeof(T) * (count ? count : 1));
+    }
+};
+
+// The tensor-core form of a level (ground_truth_tc.cuh): its operands and
+// scratch.  From kTcLeast points a level; below, the launches cost as much.
+constexpr uint64_t kTcLeast = 8192;
+struct TcLevel {
+    const void *B, *Q;
+    int dtype;
+    uint32_t d, nq, nblk, qper, qgroups;
+    int sms;
+    bool on;
+    uint32_t state[2] = {0u, 0u};          // copy of flags: values out of the filter's range, a wait gave up
+    DArr<unsigned char> qtiles, ptiles;
+    DArr<float> pnorm, lim, qq;
+    DArr<uint32_t> flags;
+
+    TcLevel(const void *base, const void *queries, int dt, uint32_t dim, uint32_t count, int sm)
+        : B(base), Q(queries), dtype(dt), d(dim), nq(count), sms(sm)
+    {
+        nblk = (d + 15u) / 16u * (dt == 2 ? 2u : 1u);
+        on = nblk <= gt_tc::kMaxBlocks;
+        qper = nblk <= 8u ? 256u : 128u;
+        qgroups = (nq + qper - 1u) / qper;
+    }
+    cudaError_t prepare(uint64_t n, cudaStream_t st)
+    {
+        if (!on || n < kTcLeast) {
+            on = false;
+            return cudaSuccess;
+        }
+        const uint32_t qt = (nq + gt_tc::kTileP - 1u) / gt_tc::kTileP;
+        const uint64_t pt = ((n < gt_tc::kTcPoints ? n : gt_tc::kTcPoints) + gt_tc::kTileP - 1u) / gt_tc::kTileP;
+        cudaError_t e;
+        if ((e = qtiles.alloc(static_cast<uint64_t>(qt) * nblk * gt_tc::kBlock)) != cudaSuccess) return e;
+        if ((e = ptiles.alloc(pt * nblk * gt_tc::kBlock)) != cudaSuccess) return e;
+        if ((e = pnorm.alloc(pt * gt_tc::kTileP)) != cudaSuccess) return e;
+        if ((e = lim.alloc(nq)) != cudaSuccess) return e;
+        if ((e = qq.alloc(nq)) != cudaSuccess) return e;
+        if ((e = flags.alloc(2)) != cudaSuccess) return e;
+        if ((e = cudaMemsetAsync(flags.p, 0, 8, st)) != cudaSuccess) return e;
+        const int smem = static_cast<int>(gt_tc::smem_bytes(nblk));
+        e = dtype == 2 ? cudaFuncSetAttribute(gt_tc::collect_tc<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem)
+                       : cudaFuncSetAttribute(gt_tc::collect_tc<0>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+        if (e != cudaSuccess) return e;
+        gt_tc::convert<<<qt, gt_tc::kTileP, 0, st>>>(Q, dtype, d, nblk, 0, nq, 1, qtiles.p, nullptr, flags.p);
+        return cudaGetLastError();
+    }
+    // Appends every pair of the level within its query's threshold (g.cnt zeroed).
+    cudaError_t collect(const GtArgs &g, cudaStream_t st)
+    {
+        gt_tc::limits<<<(nq + 127u) / 128u, 128, 0, st>>>(Q, dtype, d, nq, g.thr, lim.p, qq.p);
+        gt_tc::TcArgs a;
+        std::memset(&a, 0, sizeof a);
+        a.base = B; a.queries = Q; a.dtype = dtype; a.d = d; a.nblk = nblk; a.nq = nq; a.stride = g.stride;
+        a.ptiles = ptiles.p; a.qtiles = qtiles.p; a.pnorm = pnorm.p; a.lim = lim.p; a.qq = qq.p; a.thr = g.thr;
+        a.cnt = g.cnt; a.cd = g.cd; a.ci = g.ci; a.cap = g.cap; a.err = flags.p + 1;
+        const uint32_t smem = gt_tc::smem_bytes(nblk);
+        for (uint64_t first = 0; first < g.n; first += gt_tc::kTcPoints) {
+            a.first = first;
+            a.count = g.n - first < gt_tc::kTcPoints ? g.n - first : gt_tc::kTcPoints;
+            const uint32_t nt = static_cast<uint32_t>((a.count + gt_tc::kTileP - 1u) / gt_tc::kTileP);
+            gt_tc::convert<<<nt, gt_tc::kTileP, 0, st>>>(B, dtype, d, nblk, first, a.count, g.stride, ptiles.p, pnorm.p, flags.p);
+            // shares of the tiles: of the counts that give up to 8 blocks an SM,
+            // the one whose last wave leaves the fewest tiles waiting
+            uint32_t best = 1;
+            uint64_t cost = ~0ull;
+            for (uint32_t x = 1; x <= nt && static_cast<uint64_t>(x) * qgroups <= 8ull * sms + qgroups; ++x) {
+                const uint64_t waves = (static_cast<uint64_t>(x) * qgroups + sms - 1u) / sms;
+                const uint64_t t = waves * ((nt + x - 1u) / x + 4u);     // a block's start costs about 4 tiles
+                if (t < cost) { cost = t; best = x; }
+            }
+            a.tiles_per_cta = (nt + best - 1u) / best;
+            const dim3 grid((nt + a.tiles_per_cta - 1u) / a.tiles_per_cta, qgroups);
+            if (dtype == 2) gt_tc::collect_tc<1><<<grid, gt_tc::kThreads, smem, st>>>(a);
+            else gt_tc::collect_tc<0><<<grid, gt_tc::kThreads, smem, st>>>(a);
+            const cudaError_t e = cudaGetLastError();
+            if (e != cudaSuccess) return e;
+        }
+        return cudaSuccess;
     }
 };
 
@@ -441,6 +584,8 @@ extern "C" int bang_ground_truth(int device, const void *base, const void *queri
     const uint32_t gx = static_cast<uint32_t>((static_cast<uint64_t>(sms) * 8 + tiles - 1) / tiles) + 1;
     std::vector<uint32_t> c(nq);
     uint64_t cap = 0;
+    TcLevel tc(B, Q, dtype, d, nq, sms);
+    GT_TRY(tc.prepare(n, st));
     for (uint64_t seen = g.n;; seen = g.n) {
         g.n = seen < n / kLevel ? seen * kLevel : n;     // the last level takes every point
         g.stride = n / g.n;
@@ -456,10 +601,18 @@ extern "C" int bang_ground_truth(int device, const void *base, const void *queri
             g.cd = cd.p;
             g.ci = ci.p;
             g.cap = cap;
-            collect<<<dim3(gx, tiles), 256, tileq * d * esz, st>>>(g);
+            if (tc.on && g.n >= kTcLeast) GT_TRY(tc.collect(g, st));
+            else collect<<<dim3(gx, tiles), 256, tileq * d * esz, st>>>(g);
             GT_TRY(cudaGetLastError());
             GT_TRY(cudaMemcpyAsync(c.data(), cnt.p, nq * 4, cudaMemcpyDeviceToHost, st));
+            if (tc.on) GT_TRY(cudaMemcpyAsync(tc.state, tc.flags.p, sizeof tc.state, cudaMemcpyDeviceToHost, st));
             GT_TRY(cudaStreamSynchronize(st));
+            if (tc.on && tc.state[1]) return gtfail(BANG_ETIMEOUT, "bang_ground_truth: a tensor-core wait gave up");
+            if (tc.on && tc.state[0]) {          // values the filter cannot bound: this level again without it
+                tc.on = false;
+                --attempt;
+                continue;
+            }
             room = *std::max_element(c.begin(), c.end());
             if (room <= cap) break;
             if (attempt == 1) return gtfail(BANG_ECUDA, "bang_ground_truth: candidate lists kept growing");
@@ -475,7 +628,7 @@ extern "C" int bang_ground_truth(int device, const void *base, const void *queri
     }
     g.out_ids = dev_out ? out_ids : oids.p;
     g.out_dist = dev_out ? out_dist : odist.p;
-    select_k<<<(nq + 3) / 4, 128, 0, st>>>(g);
+    select_k<<<(nq + kKthWarps - 1) / kKthWarps, kKthWarps * kW, 0, st>>>(g);
     GT_TRY(cudaGetLastError());
     if (!dev_out) {
         GT_TRY(cudaMemcpyAsync(out_ids, oids.p, static_cast<uint64_t>(nq) * k * 4, cudaMemcpyDeviceToHost, st));

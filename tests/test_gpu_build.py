@@ -158,6 +158,39 @@ def test_ground_truth_levels(dt, d, n, k):
     assert (ids == ref_ids).all() and (dist == ref_dist).all()
 
 
+@pytest.mark.parametrize("dt,d,n,nq,k,what", [
+    ("u8", 128, 20_000, 300, 100, "any"),      # eight blocks a tile, two query groups
+    ("u8", 130, 9_000, 129, 10, "any"),        # nine blocks: 128 queries a block
+    ("u8", 256, 8_192, 5, 20, "largest"),      # the largest sums
+    ("u8", 257, 9_000, 5, 20, "any"),          # too wide for the tensor cores
+    ("i8", 100, 70_001, 257, 17, "any"),       # ragged tiles and rows
+    ("i8", 1, 8_500, 3, 256, "any"),
+    ("f32", 96, 30_000, 140, 37, "unit"),
+    ("f32", 128, 8_193, 20, 5, "offset"),      # norms far above the distances
+    ("f32", 128, 8_193, 20, 5, "huge"),        # outside the filter's range
+    ("f32", 65, 12_345, 20, 5, "tiny"),
+    ("f32", 129, 9_000, 20, 5, "unit"),
+])
+def test_ground_truth_on_the_tensor_cores(dt, d, n, nq, k, what):
+    rng = np.random.default_rng(d * 3 + n)
+    if dt == "f32":
+        X, Q = rng.normal(size=(n, d)), rng.normal(size=(nq, d))
+        f, o = {"unit": (1.0, 0.0), "offset": (1.0, 50.0), "huge": (1e18, 0.0), "tiny": (1e-22, 0.0)}[what]
+        X, Q = (X * f + o).astype(np.float32), (Q * f + o).astype(np.float32)
+    elif dt == "i8":
+        X, Q = (rng.integers(-128, 128, size=(m, d)).astype(np.int8) for m in (n, nq))
+    else:
+        lo = 250 if what == "largest" else 0
+        X, Q = (rng.integers(lo, 256, size=(m, d)).astype(np.uint8) for m in (n, nq))
+        if what == "largest":
+            Q[0] = 0
+    ids_o, dist_o = oracle.bruteforce_knn(X, Q, k)
+    ids, dist = bang.bang_ground_truth(X, Q, k)
+    assert (ids == ids_o).all()
+    fin = np.isfinite(dist_o)
+    assert (np.isfinite(dist) == fin).all() and (dist[fin] == dist_o[fin]).all()
+
+
 @pytest.mark.parametrize("dt,d,M,ns,what", [
     ("u8", 5, 5, 1001, "few values"),      # 1-wide subspaces, distance ties everywhere
     ("u8", 34, 16, 2999, "few values"),    # 3- and 2-wide
