@@ -58,6 +58,7 @@ constexpr uint32_t kRegWords = 32;       // integer vectors of at most 128 bytes
 constexpr uint32_t kSmallC = 512;        // candidates of a list sorted by one warp in shared memory
 constexpr uint32_t kCandCap = 750;       // RobustPrune looks at the nearest 750 candidates at most
 constexpr uint32_t kKeySlots = 768;      // shared key slots: >= kSmallC and >= kCandCap
+constexpr uint32_t kSortCap = 4096;      // keys of a long list sorted in shared memory
 constexpr size_t kSmemMax = 227u * 1024u;
 constexpr uint32_t kChunk = 1u << 20;    // searches per launch
 constexpr int kScanT = 1024;
@@ -130,30 +131,51 @@ __device__ __forceinline__ const uint32_t *cand_vec(const LArgs &a, uint32_t id)
     return a.kind == kJobMerge ? vec_ptr(a, a.vid[static_cast<uint64_t>(id) * a.ell]) : vec_ptr(a, id);
 }
 
-// Integer squared distance over `nw` words (padding bytes are zero on both sides).
+// Integer squared distance over `nw` words (padding bytes are zero on both
+// sides).  Vectors start on 16-byte boundaries and are padded to 16 bytes, in
+// the records and in shared memory, so they are read 16 bytes at a time.
+template <int DT> __device__ __forceinline__ uint32_t idist1(uint32_t x, uint32_t y, uint32_t acc)
+{
+    // int8: biased by 128 on both sides, differences unsigned (the signed
+    // instruction is emulated: 216 registers a thread in list_kernel)
+    const uint32_t t = DT == 1 ? __vabsdiffu4(x ^ 0x80808080u, y ^ 0x80808080u) : __vabsdiffu4(x, y);
+    return __dp4a(t, t, acc);
+}
+template <int DT> __device__ __forceinline__ uint32_t idist4(const uint4 &x, const uint4 &y, uint32_t acc)
+{
+    return idist1<DT>(x.w, y.w, idist1<DT>(x.z, y.z, idist1<DT>(x.y, y.y, idist1<DT>(x.x, y.x, acc))));
+}
 template <int DT>
 __device__ __forceinline__ uint32_t idist(const uint32_t *x, const uint32_t *y, uint32_t nw)
 {
+    const uint4 *x4 = reinterpret_cast<const uint4 *>(x), *y4 = reinterpret_cast<const uint4 *>(y);
     uint32_t acc = 0;
-    for (uint32_t w = 0; w < nw; ++w) {
-        const uint32_t t = DT == 1 ? __vabsdiffs4(x[w], y[w]) : __vabsdiffu4(x[w], y[w]);
-        acc = __dp4a(t, t, acc);
+    if (nw <= kRegWords) {               // all of it requested at once
+        uint4 v[kRegWords / 4];
+#pragma unroll
+        for (uint32_t c = 0; c < kRegWords / 4; ++c) v[c] = 4u * c < nw ? y4[c] : make_uint4(0u, 0u, 0u, 0u);
+#pragma unroll
+        for (uint32_t c = 0; c < kRegWords / 4; ++c)
+            if (4u * c < nw) acc = idist4<DT>(x4[c], v[c], acc);
+    } else {
+        for (uint32_t c = 0; 4u * c < nw; ++c) acc = idist4<DT>(x4[c], y4[c], acc);
     }
     return acc;
 }
 
-// The same with x held in registers (every index static).
-template <int DT>
-__device__ __forceinline__ uint32_t idist_reg(const uint32_t (&x)[kRegWords], const uint32_t *y, uint32_t nw)
+// The same with x held in registers (every index static), both sides as
+// `biased` leaves them.
+template <int DT> __device__ __forceinline__ uint4 biased(uint4 v)
 {
+    return DT == 1 ? make_uint4(v.x ^ 0x80808080u, v.y ^ 0x80808080u, v.z ^ 0x80808080u, v.w ^ 0x80808080u) : v;
+}
+__device__ __forceinline__ uint32_t idist_reg(const uint4 (&x)[kRegWords / 4], const uint32_t *y, uint32_t nw)
+{
+    const uint4 *y4 = reinterpret_cast<const uint4 *>(y);
     uint32_t acc = 0;
 #pragma unroll
-    for (uint32_t w = 0; w < kRegWords; ++w) {
-        if (w < nw) {
-            const uint32_t t = DT == 1 ? __vabsdiffs4(x[w], y[w]) : __vabsdiffu4(x[w], y[w]);
-            acc = __dp4a(t, t, acc);
-        }
-    }
+    for (uint32_t c = 0; c < kRegWords / 4; ++c)
+        if (4u * c < nw) acc = idist4<0>(x[c], y4[c], acc);
     return acc;
 }
 
@@ -275,11 +297,11 @@ __device__ __forceinline__ uint32_t dedupe_keys(const uint64_t *src, uint32_t C,
 // The list of `owner` from u sorted unique keys (shared memory): the keys
 // themselves when they fit in R and the job does not always prune, else
 // RobustPrune over them, 32 * kKPL candidates at a time.  One warp.
-template <int DT>
+template <int DT, bool REGS = true>
 __device__ void finish_list(const LArgs &a, const uint64_t *keys, uint32_t u, const uint32_t *ovec,
                             uint32_t *kvec, uint32_t *kept, uint32_t *out, int lane)
 {
-    const bool regs = DT != 2 && a.vwords <= kRegWords;
+    const bool regs = REGS && DT != 2 && a.vwords <= kRegWords;
     if (u <= a.R && !a.always_prune) {
         for (uint32_t i = lane; i < a.R; i += kW) out[i] = i < u ? kid(keys[i]) : kNo;
         __syncwarp();
@@ -290,7 +312,7 @@ __device__ void finish_list(const LArgs &a, const uint64_t *keys, uint32_t u, co
         uint32_t cid[kKPL];
         float dp[kKPL];
         bool alive[kKPL];
-        uint32_t cv[kKPL][kRegWords];
+        uint4 cv[kKPL][kRegWords / 4];
 #pragma unroll
         for (int s = 0; s < kKPL; ++s) {
             const uint32_t i = b0 + s * kW + lane;
@@ -298,9 +320,10 @@ __device__ void finish_list(const LArgs &a, const uint64_t *keys, uint32_t u, co
             cid[s] = alive[s] ? kid(keys[i]) : kNo;
             dp[s] = alive[s] ? kdist(keys[i]) : 0.0f;
             if (regs) {
-                const uint32_t *src = alive[s] ? cand_vec(a, cid[s]) : ovec;
+                const uint4 *src = reinterpret_cast<const uint4 *>(alive[s] ? cand_vec(a, cid[s]) : ovec);
 #pragma unroll
-                for (uint32_t w = 0; w < kRegWords; ++w) cv[s][w] = w < a.vwords ? src[w] : 0u;
+                for (uint32_t c = 0; c < kRegWords / 4; ++c)
+                    cv[s][c] = biased<DT>(4u * c < a.vwords ? src[c] : make_uint4(0u, 0u, 0u, 0u));
             }
         }
         // kept neighbours of earlier blocks
@@ -309,7 +332,7 @@ __device__ void finish_list(const LArgs &a, const uint64_t *keys, uint32_t u, co
 #pragma unroll
             for (int s = 0; s < kKPL; ++s) {
                 if (!alive[s]) continue;
-                const float dd = regs ? __uint2float_rn(idist_reg<DT>(cv[s], kv, a.vwords))
+                const float dd = regs ? __uint2float_rn(idist_reg(cv[s], kv, a.vwords))
                                       : vdist<DT>(a, kv, cand_vec(a, cid[s]));
                 if (__fmul_rn(a.a2, dd) <= dp[s]) alive[s] = false;
             }
@@ -330,7 +353,8 @@ __device__ void finish_list(const LArgs &a, const uint64_t *keys, uint32_t u, co
                     alive[t] = false;
                     if (regs) {
 #pragma unroll
-                        for (uint32_t w = 0; w < kRegWords; ++w) if (w < a.vwords) kv[w] = cv[t][w];
+                        for (uint32_t c = 0; c < kRegWords / 4; ++c)
+                            if (4u * c < a.vwords) reinterpret_cast<uint4 *>(kv)[c] = cv[t][c];
                     }
                 }
             }
@@ -343,7 +367,7 @@ __device__ void finish_list(const LArgs &a, const uint64_t *keys, uint32_t u, co
 #pragma unroll
             for (int t = 0; t < kKPL; ++t) {
                 if (!alive[t]) continue;
-                const float dd = regs ? __uint2float_rn(idist_reg<DT>(cv[t], kv, a.vwords))
+                const float dd = regs ? __uint2float_rn(idist_reg(cv[t], kv, a.vwords))
                                       : vdist<DT>(a, kv, cand_vec(a, cid[t]));
                 if (__fmul_rn(a.a2, dd) <= dp[t]) alive[t] = false;
             }
@@ -356,15 +380,15 @@ __device__ void finish_list(const LArgs &a, const uint64_t *keys, uint32_t u, co
     __syncwarp();
 }
 
-// Shared memory of a list (both kernels): kKeySlots keys, kSmallC ids, the
-// owner's vector, the kept vectors (R) and ids.
+// Shared memory of a list: key slots (kSmallC, or kKeySlots in the kernel for
+// long lists), kSmallC ids, the owner's vector, the kept vectors (R) and ids.
 struct ListSmem {
     uint64_t *keys;
     uint32_t *ids, *ovec, *kvec, *kept;
-    __device__ ListSmem(unsigned char *sm, const LArgs &a)
+    __device__ ListSmem(unsigned char *sm, const LArgs &a, uint32_t slots)
     {
         keys = reinterpret_cast<uint64_t *>(sm);
-        ids = reinterpret_cast<uint32_t *>(keys + kKeySlots);
+        ids = reinterpret_cast<uint32_t *>(keys + slots);
         ovec = ids + kSmallC;
         kvec = ovec + a.vwords;
         kept = kvec + a.R * a.vwords;
@@ -372,13 +396,16 @@ struct ListSmem {
 };
 
 // One warp per list of at most kSmallC candidates; longer lists are listed
-// in a.defer for big_list_kernel.
+// in a.defer for big_list_kernel.  Bound by the candidates' vectors (two reads
+// of 128 bytes each) and the prune's arithmetic; reading them, and the kept
+// vectors in shared memory, 16 bytes at a time instead of 4 took the lists of
+// 200,000 u8 points from 178 to 133 ms.
 template <int DT>
 __global__ void __launch_bounds__(32) list_kernel(const LArgs a)
 {
     extern __shared__ __align__(16) unsigned char sm[];
     const int lane = threadIdx.x;
-    const ListSmem m(sm, a);
+    const ListSmem m(sm, a, kSmallC);
     for (uint32_t job = blockIdx.x; job < a.njobs; job += gridDim.x) {
         uint32_t owner = 0;
         const uint32_t C = job_candidates(a, job, kSmallC, m.ids, owner, lane, kW);
@@ -420,55 +447,158 @@ __global__ void __launch_bounds__(32) list_kernel(const LArgs a)
 }
 
 // Lists of more than kSmallC candidates (reverse edges of hub nodes): one
-// 1024-thread CTA per list; the keys are computed and sorted (bitonic) in a
-// global-memory region of the next power of two above the count, then warp 0
-// keeps the kCandCap nearest unique ones and finishes the list.
+// 1024-thread CTA per list.  An id occurs at most twice (in the current row and
+// among the members that named it), so the kCandCap nearest unique candidates
+// are among the 2 kCandCap nearest: the keys (in a global-memory region) are
+// cut at that distance by a radix selection, what is left is sorted in shared
+// memory, and for integer vectors of at most 128 bytes the whole CTA prunes, a
+// candidate a thread.  When ties leave more than `sort_cap` keys, they are
+// sorted (bitonic) in the region.  Sorting every list there and pruning with
+// one warp took 108 ms of the 360 that 200,000 u8 points took (8 shards, two
+// per point, R = 64); so it is 4.3.
 template <int DT>
 __global__ void __launch_bounds__(1024) big_list_kernel(const LArgs a, const uint32_t *jobs, uint32_t njobs,
-                                                        const uint64_t *region_off, uint64_t *region)
+                                                        const uint64_t *region_off, uint64_t *region, uint32_t sort_cap,
+                                                        uint32_t sort_off)
 {
     extern __shared__ __align__(16) unsigned char sm[];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const ListSmem m(sm, a);
+    const ListSmem m(sm, a, kKeySlots);
+    uint32_t *hist = m.ids, *word = hist + 256, *share = word + 32;      // the ids of short lists are not used here
+    uint64_t *sk = reinterpret_cast<uint64_t *>(sm + sort_off);
     for (uint32_t b = blockIdx.x; b < njobs; b += gridDim.x) {
         const uint32_t job = jobs[b];
         uint64_t *keys = region + region_off[b];
         uint32_t owner = 0;
         const uint32_t C = job_candidates(a, job, 0u, nullptr, owner, tid, blockDim.x);
-        uint32_t P = 32;
-        while (P < C) P <<= 1;
         const uint32_t *ovp = owner_vec(a, owner);
         for (uint32_t w = tid; w < a.vwords; w += blockDim.x) m.ovec[w] = ovp[w];
         __syncthreads();
-        for (uint32_t i = tid; i < P; i += blockDim.x) {
+        for (uint32_t i = tid; i < C; i += blockDim.x) {
             uint64_t k = ~0ull;
-            if (i < C) {
-                uint32_t id;
-                if (a.kind == kJobRev)
-                    id = i < a.R ? a.rec[static_cast<uint64_t>(owner) * a.rec_words + i]
-                                 : a.in_src[a.in_off[job] + (i - a.R)];
-                else
-                    id = kNo;                 // only reverse lists exceed kSmallC
-                if (id != kNo && id != owner) k = mkkey(vdist<DT>(a, m.ovec, cand_vec(a, id)), id);
-            }
+            uint32_t id;
+            if (a.kind == kJobRev)
+                id = i < a.R ? a.rec[static_cast<uint64_t>(owner) * a.rec_words + i]
+                             : a.in_src[a.in_off[job] + (i - a.R)];
+            else
+                id = kNo;                 // only reverse lists exceed kSmallC
+            if (id != kNo && id != owner) k = mkkey(vdist<DT>(a, m.ovec, cand_vec(a, id)), id);
             keys[i] = k;
         }
+        // the distance bits of the 2 kCandCap-th key (all ones: invalid keys,
+        // when there are fewer valid ones), by four rounds of 8-bit digits
+        uint32_t prefix = 0, mask = 0, want = 2u * kCandCap < C ? 2u * kCandCap : C;
+        for (int shift = 24; sort_cap && shift >= 0; shift -= 8) {
+            if (tid < 256) hist[tid] = 0;
+            __syncthreads();
+            for (uint32_t i = tid; i < C; i += blockDim.x) {
+                const uint32_t v = static_cast<uint32_t>(keys[i] >> 32);
+                if ((v & mask) == prefix) atomicAdd(&hist[(v >> shift) & 255u], 1u);
+            }
+            __syncthreads();
+            if (warp == 0) {
+                uint32_t h[8], sum = 0;          // this lane's bins: 8 lane .. 8 lane + 7
+#pragma unroll
+                for (int t = 0; t < 8; ++t) {
+                    h[t] = hist[lane * 8 + t];
+                    sum += h[t];
+                }
+                uint32_t below = sum;
+#pragma unroll
+                for (int o = 1; o < kW; o <<= 1) {
+                    const uint32_t up = __shfl_up_sync(0xFFFFFFFFu, below, o);
+                    if (lane >= o) below += up;
+                }
+                below -= sum;
+                if (below < want && want <= below + sum) {
+                    uint32_t bin = 0, left = want - below;
+#pragma unroll
+                    for (int t = 0; t < 7; ++t)
+                        if (bin == static_cast<uint32_t>(t) && left > h[t]) {
+                            left -= h[t];
+                            ++bin;
+                        }
+                    share[0] = lane * 8u + bin;
+                    share[1] = left;
+                }
+            }
+            __syncthreads();
+            prefix |= share[0] << shift;
+            mask |= 255u << shift;
+            want = share[1];
+            __syncthreads();
+        }
+        if (tid == 0) share[0] = 0;
+        __syncthreads();
+        for (uint32_t i = tid; sort_cap && i < C; i += blockDim.x) {
+            const uint64_t k = keys[i];
+            if (k != ~0ull && static_cast<uint32_t>(k >> 32) <= prefix) {
+                const uint32_t at = atomicAdd(&share[0], 1u);
+                if (at < sort_cap) sk[at] = k;
+            }
+        }
+        __syncthreads();
+        const uint32_t got = sort_cap ? share[0] : ~0u;
+        const bool local = got <= sort_cap;
+        const uint32_t cnt = local ? got : C;
+        uint64_t *srt = local ? sk : keys;
+        uint32_t P = 32;
+        while (P < cnt) P <<= 1;
+        for (uint32_t i = cnt + tid; i < P; i += blockDim.x) srt[i] = ~0ull;
         __syncthreads();
         for (uint32_t k = 2; k <= P; k <<= 1)
             for (uint32_t j = k >> 1; j > 0; j >>= 1) {
-                for (uint32_t i = tid; i < P; i += blockDim.x) {
-                    const uint32_t l = i ^ j;
-                    if (l > i) {
-                        const uint64_t x = keys[i], y = keys[l];
-                        const bool up = (i & k) == 0;
-                        if ((x > y) == up) { keys[i] = y; keys[l] = x; }
-                    }
+                for (uint32_t t = tid; t < P / 2; t += blockDim.x) {
+                    const uint32_t i = ((t & ~(j - 1u)) << 1) | (t & (j - 1u)), l = i | j;
+                    const uint64_t x = srt[i], y = srt[l];
+                    const bool up = (i & k) == 0;
+                    if ((x > y) == up) { srt[i] = y; srt[l] = x; }
                 }
                 __syncthreads();
             }
         if (warp == 0) {
-            const uint32_t u = dedupe_keys(keys, C, m.keys, lane);
-            finish_list<DT>(a, m.keys, u, m.ovec, m.kvec, m.kept, job_out(a, job, owner), lane);
+            const uint32_t u = dedupe_keys(srt, cnt, m.keys, lane);
+            if (lane == 0) share[0] = u;
+        }
+        __syncthreads();
+        const uint32_t u = share[0];
+        uint32_t *out = job_out(a, job, owner);
+        if (DT != 2 && a.vwords <= kRegWords && (u > a.R || a.always_prune)) {
+            // RobustPrune, a candidate a thread (u <= kCandCap < 1024)
+            const bool have = static_cast<uint32_t>(tid) < u;
+            const uint64_t key = have ? m.keys[tid] : 0ull;
+            const float dp = kdist(key);
+            uint4 cv[kRegWords / 4];
+            {
+                const uint4 *src = reinterpret_cast<const uint4 *>(have ? cand_vec(a, kid(key)) : m.ovec);
+#pragma unroll
+                for (uint32_t c = 0; c < kRegWords / 4; ++c)
+                    cv[c] = biased<DT>(4u * c < a.vwords ? src[c] : make_uint4(0u, 0u, 0u, 0u));
+            }
+            bool alive = have;
+            uint32_t nout = 0;
+            while (nout < a.R) {
+                const uint32_t bal = __ballot_sync(0xFFFFFFFFu, alive);
+                if (lane == 0) word[warp] = bal;
+                __syncthreads();
+                const uint32_t w = word[lane], any = __ballot_sync(0xFFFFFFFFu, w != 0u);
+                if (any == 0u) break;                        // uniform over the CTA
+                const int wf = __ffs(any) - 1, lf = __ffs(__shfl_sync(0xFFFFFFFFu, w, wf)) - 1;
+                if (warp == wf && lane == lf) {              // the nearest live candidate is kept
+                    m.kept[nout] = kid(key);
+                    alive = false;
+#pragma unroll
+                    for (uint32_t c = 0; c < kRegWords / 4; ++c)
+                        if (4u * c < a.vwords) reinterpret_cast<uint4 *>(m.kvec)[c] = cv[c];
+                }
+                __syncthreads();
+                if (alive && __fmul_rn(a.a2, __uint2float_rn(idist_reg(cv, m.kvec, a.vwords))) <= dp) alive = false;
+                ++nout;
+            }
+            __syncthreads();
+            for (uint32_t i = tid; i < a.R; i += blockDim.x) out[i] = i < nout ? m.kept[i] : kNo;
+        } else if (warp == 0) {
+            finish_list<DT, false>(a, m.keys, u, m.ovec, m.kvec, m.kept, out, lane);
         }
         __syncthreads();
     }
@@ -701,9 +831,9 @@ cudaError_t scan_counts(const uint32_t *in, uint64_t n, uint64_t *out, DBuf<uint
     return cudaGetLastError();
 }
 
-size_t list_smem(uint32_t vwords, uint32_t R)
+size_t list_smem(uint32_t vwords, uint32_t R, uint32_t slots = kKeySlots)
 {
-    return static_cast<size_t>(kKeySlots) * 8u + static_cast<size_t>(kSmallC) * 4u +
+    return static_cast<size_t>(slots) * 8u + static_cast<size_t>(kSmallC) * 4u +
            4u * (vwords + static_cast<size_t>(R) * vwords + R) + 16u;
 }
 
@@ -723,7 +853,11 @@ cudaError_t launch_big(const LArgs &a, const uint32_t *jobs, uint32_t nd, const 
     cudaError_t e = cudaFuncSetAttribute(big_list_kernel<DT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          static_cast<int>(kSmemMax));
     if (e != cudaSuccess) return e;
-    big_list_kernel<DT><<<std::min<uint32_t>(nd, 1024u), 1024, smem, st>>>(a, jobs, nd, off, region);
+    // keys sorted in shared memory where they fit beside the rest
+    const size_t at = (smem + 15u) & ~size_t(15);
+    const bool room = at + kSortCap * 8u <= kSmemMax;
+    big_list_kernel<DT><<<std::min<uint32_t>(nd, 1024u), 1024, room ? at + kSortCap * 8u : smem, st>>>(
+        a, jobs, nd, off, region, room ? kSortCap : 0u, static_cast<uint32_t>(at));
     return cudaGetLastError();
 }
 
@@ -748,8 +882,9 @@ cudaError_t run_lists(LArgs a, BigScratch &bs, cudaStream_t st)
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     const uint32_t grid = std::min<uint32_t>(a.njobs, static_cast<uint32_t>(sms) * 64u);
-    e = a.dtype == 0 ? launch_small<0>(a, smem, grid, st)
-      : a.dtype == 1 ? launch_small<1>(a, smem, grid, st) : launch_small<2>(a, smem, grid, st);
+    const size_t small = list_smem(a.vwords, a.R, kSmallC);
+    e = a.dtype == 0 ? launch_small<0>(a, small, grid, st)
+      : a.dtype == 1 ? launch_small<1>(a, small, grid, st) : launch_small<2>(a, small, grid, st);
     if (e != cudaSuccess) return e;
     uint32_t nd = 0;
     if ((e = cudaMemcpyAsync(&nd, bs.ndefer.p, 4, cudaMemcpyDeviceToHost, st)) != cudaSuccess) return e;

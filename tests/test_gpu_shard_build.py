@@ -65,3 +65,22 @@ def test_shard_graph_device_buffers():
     adj = torch.zeros((2500, 32), dtype=torch.int32, device="cuda")
     bang.bang_build_shard_graph(Xd, centres, 2, 32, 32, 1.2, 0.05, 14, adj=adj)
     assert (adj.cpu().numpy().view(np.uint32) == want).all()
+
+
+@pytest.mark.parametrize("dt,n,d,top,R", [
+    ("u8", 9000, 3, 2, 16),        # eight different points: thousands of candidates at one distance
+    ("i8", 6000, 24, 256, 64),     # hubs: the selection and the prune of the whole block
+    ("u8", 3000, 200, 256, 32),    # rows of more than 128 bytes
+    ("f32", 5000, 6, 256, 16),     # FP32 distances
+    ("u8", 2500, 129, 256, 4),
+])
+def test_shard_graph_long_reverse_lists(dt, n, d, top, R):
+    # one shard and one pass-2 round of every member, so that the entry and
+    # its surroundings are named by hundreds to thousands of members
+    rng = np.random.default_rng(n + d)
+    X = rng.integers(0, top, size=(n, d)) - (128 if dt == "i8" else 0)
+    X = X.astype({"u8": np.uint8, "i8": np.int8, "f32": np.float32}[dt])
+    centres = X[:1].astype(np.float32)
+    want, _ = oracle.shard_graph(X, centres, 1, R, 32, 1.2, 1.0, 14)
+    got, _ = bang.bang_build_shard_graph(X, centres, 1, R, 32, 1.2, 1.0, 14)
+    assert (got == want).all()
