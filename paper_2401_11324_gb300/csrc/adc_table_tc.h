@@ -24,6 +24,7 @@ struct TcTableArgs {
     void *out;                  // device, nq*M*256 FP32 or BF16
     uint32_t out_bf16;
     uint32_t tf32;              // queries rounded to TF32 (pair with the TF32 centroid tiles)
+    uint32_t nbmax;             // most K blocks a subspace spans (set by launch_tc_tables)
     unsigned int *err;          // device flag, set to 1 if a wait gave up
 };
 

@@ -130,3 +130,39 @@ def test_fp32_searches_on_tensor_core_tables():
     assert abs(rec[1] - rec[0]) <= 0.005 + 1.0 / (10 * len(Q))
     assert rec[2] >= rec[0] - 0.1
     ix.close()
+
+
+@pytest.mark.parametrize("dt", ["u8", "i8", "f32"])
+@pytest.mark.parametrize("d,M,nq", [(128, 32, 1), (130, 32, 127), (97, 30, 129), (64, 1, 257),
+                                    (48, 2, 128), (33, 33, 40)])
+def test_tables_at_the_edges_of_their_tiles(dt, d, M, nq):
+    # queries around a tile of 128, subspaces that span one to four blocks of 16
+    # dimensions or share one, the last group of subspaces not full
+    rng = np.random.default_rng(d + M + nq)
+    if dt == "f32":
+        X, Q = (rng.normal(size=(m, d)).astype(np.float32) for m in (300, nq))
+    else:
+        lo, ty = (0, np.uint8) if dt == "u8" else (-128, np.int8)
+        X, Q = (rng.integers(lo, lo + 256, size=(m, d)).astype(ty) for m in (300, nq))
+    cb = rng.normal(size=256 * d).astype(np.float32) * (1.0 if dt == "f32" else 60.0)
+    cb = np.ascontiguousarray(cb, np.float32)
+    h = bang.bang_create(0)
+    bang.bang_load_pq(h, d, M, cb, np.zeros((300, M), np.uint8), 300)
+    bang.bang_register_vectors(h, X, {"u8": 0, "i8": 1, "f32": 2}[dt])
+    q = torch.from_numpy(Q).cuda()
+    off = oracle.chunk_offsets(d, M)
+    want = np.empty((nq, M, 256))
+    scale = np.empty((nq, M, 256))               # size of the cancelling terms
+    for s in range(M):
+        o, w = int(off[s]), int(off[s + 1] - off[s])
+        C = cb[256 * o:256 * (o + w)].reshape(256, w).astype(np.float64)
+        qs = Q[:, o:o + w].astype(np.float64)
+        want[:, s] = ((qs[:, None] - C[None]) ** 2).sum(2)
+        scale[:, s] = (qs ** 2).sum(1)[:, None] + (C ** 2).sum(1)[None]
+    for form, ty, extra in ((0, torch.float32, 0.0), (1, torch.bfloat16, 2.0 ** -8)):
+        out = torch.full((nq + 1, M, 256), -1.0, dtype=ty, device="cuda")
+        bang.bang_pq_tables(h, q, nq, out, form)
+        got = out.float().cpu().numpy()
+        assert (got[nq] == -1.0).all()           # nothing behind the last query's table
+        assert (np.abs(got[:nq] - want) <= 4e-6 * scale + 2e-3 + extra * want).all()
+    bang.bang_destroy(h)
