@@ -706,7 +706,8 @@ namespace {
 // bang_search_batched (k, L are the bounds; persistent launch).
 int search_impl(bang_index *ix, const void *queries, uint32_t nq, uint32_t k, uint32_t L,
                 const uint32_t *k_arr, const uint32_t *L_arr, bool persistent,
-                const bang_search_params *params, uint32_t *out_ids, float *out_dist, void *stream)
+                const bang_search_params *params, uint32_t *out_ids, float *out_dist, void *stream,
+                bool overlapped = false)
 {
     if (!ix) return fail(BANG_EINVAL, "bang_search: index is NULL");
     if (!ix->have_pq || !ix->have_graph || !ix->have_vectors)
@@ -866,6 +867,7 @@ int search_impl(bang_index *ix, const void *queries, uint32_t nq, uint32_t k, ui
     a.phase_cycles = static_cast<unsigned long long *>(dptr(7));
     a.carveout = p.smem_carveout;
     a.ntab = ntab;
+    a.overlapped = overlapped ? 1u : 0u;
     if (p.rerank != 0) {       // staged re-rank: lists sized by the iteration cap (or L)
         uint64_t cap = p.iter_cap ? p.iter_cap : 8ull * L + 64ull;
         if (cap < L) cap = L;
@@ -923,6 +925,14 @@ int search_impl(bang_index *ix, const void *queries, uint32_t nq, uint32_t k, ui
 }
 
 }  // namespace
+
+int bang::search_batched(bang_index *ix, const void *queries, uint32_t nq, const uint32_t *k_per_q,
+                         const uint32_t *L_per_q, uint32_t k_max, uint32_t L_max, const bang_search_params *params,
+                         uint32_t *out_ids, float *out_dist, void *stream, bool overlapped)
+{
+    return search_impl(ix, queries, nq, k_max, L_max, k_per_q, L_per_q, true, params, out_ids, out_dist, stream,
+                       overlapped);
+}
 
 extern "C" {
 

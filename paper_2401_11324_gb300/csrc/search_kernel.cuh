@@ -110,6 +110,7 @@ struct SearchArgs {
     uint32_t *cand_n;
     uint32_t cand_list;       // 1: the candidates are the final worklist instead (cand_cap >= L)
     uint32_t carveout;        // preferred shared-memory share of L1 in percent (0: the CUDA driver's choice)
+    uint32_t overlapped;      // other launches share the GPU (chooses the form of the search only)
     uint32_t ntab;            // kModeF32Lazy: subspaces (the first ones) whose entries stay in a table
 };
 

@@ -816,12 +816,13 @@ inline uint32_t team_expanders(const SearchArgs &a, int mode, int sms)
 {
     const uint32_t smem = ((TeamLayout(a.M, a.log2z, a.L, a.k, a.d, a.R, mode, 2).total + 127u) & ~127u) + 1024u;
     const uint32_t fit = 228u * 1024u / smem, share = (a.nq + static_cast<uint32_t>(sms) - 1u) / static_cast<uint32_t>(sms);
-    const uint32_t c = fit < share ? fit : share;
-    // a persistent launch of a few waves at most is one of several that overlap
-    // (the server's): then the SMs are full whatever its own number
-    // (served BF16, c = 7: 2,372 us with one warp, 2,428 with three expanders)
-    if (a.queue && fit > 6u && share > 2u && share < 4u * fit) return 0u;
+    // launches that overlap (the server's) fill the SMs together, and all take
+    // the same form: 24 requests, BF16 table, L up to 256 (c = 7), against one
+    // warp per query: two expanders 1.02 times as fast, three 1.06; the form
+    // chosen launch by launch, so that both kinds share the SMs, 0.92
+    const uint32_t c = a.overlapped || fit < share ? fit : share;
     uint32_t e = c > 0 ? 27u / c - (c <= 27u ? 1u : 0u) : 0u;
+    if (a.overlapped) e = c <= 7u ? 3u : 0u;
     e = e < kTeamMaxExpanders ? e : kTeamMaxExpanders;
     if (e == 3u) {       // the third slot must not cost a resident query
         const uint32_t t3 = ((TeamLayout(a.M, a.log2z, a.L, a.k, a.d, a.R, mode, 3).total + 127u) & ~127u) + 1024u;

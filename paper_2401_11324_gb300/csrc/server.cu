@@ -180,8 +180,8 @@ int start_launch(bang_server *s, Stream &st, Launch &ln)
     p.mode = s->cfg.mode;
     p.bloom_log2 = s->cfg.bloom_log2;
     p.early_codes = s->cfg.early_codes;
-    int rc = bang_search_batched(s->ix, dv.q, nq, dv.k, dv.L, s->cfg.k_max, s->cfg.L_max, &p, dv.ids,
-                                 dv.dist, st.stream);
+    int rc = bang::search_batched(s->ix, dv.q, nq, dv.k, dv.L, s->cfg.k_max, s->cfg.L_max, &p, dv.ids,
+                                  dv.dist, st.stream, true);
     if (rc != BANG_OK) return rc;
     const size_t out_bytes = 2 * up(static_cast<size_t>(nq) * s->cfg.k_max * 4);   // ids, distances
     cudaMemcpyAsync(h.ids, dv.ids, out_bytes, cudaMemcpyDeviceToHost, st.stream);
