@@ -139,10 +139,11 @@ struct SmemLayout {
         off_Ck = o;     o += up16(k > (uint32_t)kRegK && mode != kModeExact ? k * 8u : 0u);
         // table-build scratch (query, subspace offsets, 8-bit-table minima):
         // dead once the table is built, so it shares the worklist's space
-        // when that is large enough (not without a table: the loop reads it)
-        const uint32_t sq = up16(mode != kModeExact ? d * 4u : 0u), so = up16((M + 1u) * 4u),
+        // when that is large enough (not without a table: the loop reads it;
+        // exact mode: an integer query's bytes, which the loop reads)
+        const uint32_t sq = up16(mode != kModeExact ? d * 4u : 128u), so = up16(mode != kModeExact ? (M + 1u) * 4u : 0u),
                        sl = up16(mode == kModeQ8 ? M * 4u : 0u);
-        uint32_t b = !lazy && up16(L * 8u) >= sq + so + sl ? off_L : o;
+        uint32_t b = mode != kModeExact && !lazy && up16(L * 8u) >= sq + so + sl ? off_L : o;
         off_q = b;      b += sq;
         off_offs = b;   b += so;
         off_lo = b;     b += sl;
@@ -712,6 +713,7 @@ __global__ void __launch_bounds__(32) search_kernel(const SearchArgs a)
         }
         VecShare<DT, DCH> qs;
         load_share<DT, DCH>(qp, d, a.vec_ok != 0, lane, qs);
+        if (!kPQ && DT != 2 && DCH == 1) reinterpret_cast<uint32_t *>(qv)[lane] = qs.w[0];
         for (uint32_t w = lane; w < nwords; w += kWarp) bloom[w] = 0u;
         __syncwarp();
         bool table_failed = false;
@@ -932,10 +934,18 @@ __global__ void __launch_bounds__(32) search_kernel(const SearchArgs a)
             } else if (DT != 2 && DCH == 1 && (d & 15u) == 0 && a.vecb_ok) {
                 // integer data sums exactly in any order, so one lane takes
                 // one new neighbour (its whole row) and all of them are
-                // requested at once; query words come by shuffle
-                const uint32_t nw = d / 4u;  // 32-bit words per row, <= 32
-                for (uint32_t j0 = 0; j0 < nn; j0 += kWarp) {
-                    const uint32_t j = j0 + static_cast<uint32_t>(lane);
+                // requested at once; the query's words come from shared
+                // memory, 16 bytes at a time to all lanes (10,000 u8 queries
+                // at L = 48: 0.75 ms; as shuffles, one a word, and with the
+                // keys passed through shared memory, 0.82)
+                in_regs = true;
+                const uint32_t nv = d / 16u;     // 16-byte chunks per row, <= 8
+                const uint32_t bias = DT == 1 ? 0x80808080u : 0u;
+                const uint4 *q4 = reinterpret_cast<const uint4 *>(qv);
+#pragma unroll
+                for (int t = 0; t < RPL; ++t) {
+                    if (static_cast<uint32_t>(kWarp * t) >= nn) break;           // warp-uniform
+                    const uint32_t j = lane + kWarp * t;
                     const bool act = j < nn;
                     const uint32_t id = act ? Nid[j] : 0u;
                     const uint4 *row = reinterpret_cast<const uint4 *>(static_cast<const E *>(a.base) +
@@ -943,23 +953,25 @@ __global__ void __launch_bounds__(32) search_kernel(const SearchArgs a)
                     uint4 xv[8];
 #pragma unroll
                     for (int c = 0; c < 8; ++c)
-                        xv[c] = (act && 4u * c < nw) ? __ldg(row + c) : make_uint4(0u, 0u, 0u, 0u);
+                        xv[c] = (act && static_cast<uint32_t>(c) < nv) ? __ldg(row + c) : make_uint4(0u, 0u, 0u, 0u);
                     uint32_t acc = 0;
 #pragma unroll
                     for (int c = 0; c < 8; ++c) {
-                        const uint32_t xw[4] = {xv[c].x, xv[c].y, xv[c].z, xv[c].w};
+                        if (static_cast<uint32_t>(c) < nv) {
+                            const uint4 qc = q4[c];
+                            const uint32_t xw[4] = {xv[c].x ^ bias, xv[c].y ^ bias, xv[c].z ^ bias, xv[c].w ^ bias};
+                            const uint32_t qwd[4] = {qc.x, qc.y, qc.z, qc.w};
 #pragma unroll
-                        for (int i = 0; i < 4; ++i) {
-                            const uint32_t w = 4u * c + i;
-                            const uint32_t qw = __shfl_sync(0xFFFFFFFFu, qs.w[0], static_cast<int>(w));
-                            const uint32_t x = DT == 1 ? xw[i] ^ 0x80808080u : xw[i];
-                            if (w < nw) {
-                                const uint32_t df = __vabsdiffu4(qw, x);
+                            for (int i = 0; i < 4; ++i) {
+                                const uint32_t df = __vabsdiffu4(qwd[i], xw[i]);
                                 acc = __dp4a(df, df, acc);
                             }
                         }
                     }
-                    if (act) Nk[j] = make_key(acc, id);
+                    if (act) {
+                        kk[t] = make_key(acc, id);
+                        kv[t] = true;
+                    }
                 }
             } else {
                 for (uint32_t j0 = 0; j0 < nn; j0 += 4) {
