@@ -27,9 +27,9 @@
 // iteration; the waits for rows and code rows, 40 % of it there, are gone).
 // So where the entry after u* is ready too, both are expanded in one step (a
 // quarter to a third of the steps); an expander takes about 3,000 cycles, hence
-// three.  10,000 u8 queries, 1M points, L = 224, FP32 table, HBM: 6.96 -> 5.27 ms;
-// 3,000 float queries, d = 96, M = 48, L = 128: 4.23 -> 2.64 ms; one query at
-// L = 64: 169 -> 125 us.
+// three.  10,000 u8 queries, 1M points, L = 224, FP32 table, HBM: 7.04 -> 5.10 ms;
+// 3,000 float queries, d = 96, M = 48, L = 128: 4.22 -> 2.53 ms; one query at
+// L = 64: 218 -> 157 us (169 -> 125 on another day).
 //
 // Slots are handed over through two mbarriers each (request, result); every
 // wait is bounded, and a wait that gave up ends the query with status 3.
@@ -482,8 +482,9 @@ __global__ void __maxnreg__(team_regs(DCH, MODE)) team_kernel(const SearchArgs a
                     break;
                 }
                 const uint32_t u = key_id(ukey), u2 = key_id(lkey);
-                const uint32_t se = static_cast<uint32_t>(__ffs(__ballot_sync(0xFFFFFFFFu, sid == u))) - 1u;
-                const uint32_t s2 = static_cast<uint32_t>(__ffs(__ballot_sync(0xFFFFFFFFu, sid == u2))) - 1u;
+                // (one bit at most: the leading-zero count is half of __ffs)
+                const uint32_t se = 31u - __clz(__ballot_sync(0xFFFFFFFFu, sid == u));
+                const uint32_t s2 = 31u - __clz(__ballot_sync(0xFFFFFFFFu, sid == u2));     // ~0: in no slot
                 if (!team_wait(result(se), (phase >> se) & 1u)) {
                     status = 3;
                     break;
@@ -613,19 +614,18 @@ __global__ void __maxnreg__(team_regs(DCH, MODE)) team_kernel(const SearchArgs a
                                 lo += b * mm;
                             }
                             xpos = lo;
-                            for (uint32_t tt = 0; tt < nm; ++tt) xpos += Nk[tt] < x;
+                            for (uint32_t tt = 0; tt < nm; tt += 4) {            // Nk is 32 keys long
+                                const uint64_t k0 = Nk[tt], k1 = Nk[tt + 1], k2 = Nk[tt + 2], k3 = Nk[tt + 3];
+                                xpos += (k0 < x) + (tt + 1 < nm && k1 < x) + (tt + 2 < nm && k2 < x) +
+                                        (tt + 3 < nm && k3 < x);
+                            }
                         }
                         const uint32_t rmin = __reduce_min_sync(0xFFFFFFFFu, lo);
                         if (xpos < L) atomicOr(&obits[xpos >> 5], 1u << (xpos & 31u));
                         __syncwarp();
-                        const uint32_t wbits = static_cast<uint32_t>(lane) < nw ? obits[lane] : 0u;
-                        uint32_t pre = __popc(wbits);
-#pragma unroll
-                        for (int h = 1; h < kWarp; h <<= 1) {
-                            const uint32_t v = __shfl_up_sync(0xFFFFFFFFu, pre, h);
-                            if (lane >= h) pre += v;
-                        }
-                        pre -= __popc(wbits);
+                        // new keys at or below the chunk in hand: all of them,
+                        // less those of the chunks already done, from the end
+                        uint32_t upto = __popc(__ballot_sync(0xFFFFFFFFu, xpos < L));
                         const int32_t cmin = static_cast<int32_t>(rmin >> 5);
                         constexpr int kG = 4;    // chunks read before they are written
 #pragma unroll 1
@@ -638,8 +638,9 @@ __global__ void __maxnreg__(team_regs(DCH, MODE)) team_kernel(const SearchArgs a
                                 mv[g] = 0;
                                 dst[g] = 0xFFFFFFFFu;
                                 if (c >= cmin) {
-                                    const uint32_t w = __shfl_sync(0xFFFFFFFFu, wbits, c);
-                                    const uint32_t below = __shfl_sync(0xFFFFFFFFu, pre, c) + __popc(w & lt);
+                                    const uint32_t w = obits[c];
+                                    upto -= __popc(w);
+                                    const uint32_t below = upto + __popc(w & lt);
                                     const uint32_t p = static_cast<uint32_t>(c) * 32u + lane;
                                     if (p < nl2 && p >= rmin && !((w >> lane) & 1u)) {
                                         mv[g] = Lk[p - below];
