@@ -426,7 +426,7 @@ int bang_build_pq(int device, const void *base, bang_dtype dtype, uint64_t n, ui
  * sum rounded; sorted by (distance, id), padded with 0xFFFFFFFF / +inf when
  * n < k.  base (n*d) and queries (nq*d) host or device, of dtype; out_ids and
  * out_dist (nq*k) both host or both device.  k <= 256, d <= 4096.  Allocates
- * device scratch (about nq*(k*400 + 3000) bytes plus copies of host
+ * device scratch (about nq*(k*400 + 3000) bytes, up to 0.9 GB of converted rows, and copies of host
  * inputs) and blocks until done. */
 int bang_ground_truth(int device, const void *base, const void *queries, bang_dtype dtype, uint64_t n,
                       uint32_t nq, uint32_t d, uint32_t k, uint32_t *out_ids, double *out_dist,

@@ -13,16 +13,17 @@
 // query's threshold to that query's candidate list (about 16 k of them); their
 // k-th distance is the next threshold, and so on until all n points have been
 // streamed over; integer rows of up to 256 dimensions and FP32 rows of up to
-// 128 on the tensor cores (ground_truth_tc.cuh), others as above.  (3) One warp per query picks the k smallest candidates of
+// 208 on the tensor cores (ground_truth_tc.cuh), others as above.  (3) One warp per query picks the k smallest candidates of
 // the last list by (distance, id).  A list that overflows its capacity is
 // detected and its pass rerun with room for the longest list.
 //
-// Step (1) keeps each query's k nearest sorted in one warp, a serial chain per
+// Step (1) kept each query's k nearest sorted in one warp, a serial chain per
 // insertion: over 262,144 points it took 294 of 375 ms (10,000 u8 queries,
-// d = 128, 1M points, k = 100), over 1,024 it takes 2.2.  The streamed levels
-// are a contraction: with a point per thread (vabsdiff4 + dp4a) they took 73
-// ms, on the tensor cores 7.6; the sorted selection took 3.9 ms one neighbour
-// after the other, 0.1 gathered and sorted.
+// d = 128, 1M points, k = 100).  Over 1,024, with the distances in shared memory
+// and a radix selection, it takes 1.2.  The streamed levels are a contraction:
+// with a point per thread (vabsdiff4 + dp4a) they took 73 ms, on the tensor
+// cores 7.4; the sorted selection took 3.9 ms one neighbour after the other, 0.1
+// gathered and sorted.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -39,7 +40,7 @@ namespace {
 
 constexpr uint32_t kNo = 0xFFFFFFFFu;
 constexpr int kW = 32;
-constexpr int kKPL = 8;                  // top-k entries per lane in pass 1: k <= 256
+constexpr uint32_t kMaxK = 256;
 constexpr uint32_t kTileQ = 128;         // at most this many queries per CTA in pass 2
 constexpr uint32_t kSample = 1024;       // points of the first threshold
 constexpr uint32_t kLevel = 16;          // each further level streams over this many times as many
@@ -123,68 +124,6 @@ __device__ __forceinline__ bool less_pair(uint64_t da, uint32_t ia, uint64_t db,
     return da < db || (da == db && ia < ib);
 }
 
-// Step 1: one warp per query, the exact k nearest of the level's points kept
-// sorted across the warp (8 per lane); the threshold is the k-th distance.
-__global__ void sample_threshold(const GtArgs g)
-{
-    const uint64_t S = g.n;
-    const int lane = threadIdx.x & 31;
-    const uint32_t q = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    if (q >= g.nq) return;
-    const void *qr = query_row(g, q);
-    uint64_t td[kKPL];
-    uint32_t ti[kKPL];
-#pragma unroll
-    for (int t = 0; t < kKPL; ++t) { td[t] = ~0ull; ti[t] = kNo; }
-    uint32_t cnt = 0;
-    uint64_t thd = ~0ull;
-    uint32_t thi = kNo;
-    for (uint64_t b0 = 0; b0 < S; b0 += kW) {
-        const uint64_t i = b0 + lane;
-        uint64_t dk = ~0ull;
-        uint32_t ik = kNo;
-        if (i < S) {
-            dk = static_cast<uint64_t>(__double_as_longlong(dist_rows(g, qr, i * g.stride)));
-            ik = static_cast<uint32_t>(i);
-        }
-        uint32_t want = __ballot_sync(0xFFFFFFFFu, ik != kNo && less_pair(dk, ik, thd, thi));
-        while (want) {
-            const int src = __ffs(want) - 1;
-            want &= want - 1;
-            const uint64_t xd = __shfl_sync(0xFFFFFFFFu, dk, src);
-            const uint32_t xi = __shfl_sync(0xFFFFFFFFu, ik, src);
-            if (!less_pair(xd, xi, thd, thi)) continue;
-            uint32_t below = 0;
-#pragma unroll
-            for (int t = 0; t < kKPL; ++t) below += less_pair(td[t], ti[t], xd, xi) ? 1u : 0u;
-            const uint32_t pos = __reduce_add_sync(0xFFFFFFFFu, below);
-            const uint64_t cd = __shfl_up_sync(0xFFFFFFFFu, td[kKPL - 1], 1);
-            const uint32_t ci = __shfl_up_sync(0xFFFFFFFFu, ti[kKPL - 1], 1);
-#pragma unroll
-            for (int t = kKPL - 1; t >= 0; --t) {
-                const uint32_t idx = static_cast<uint32_t>(lane) * kKPL + t;
-                const uint64_t pd = t > 0 ? td[t - 1] : (lane > 0 ? cd : ~0ull);
-                const uint32_t pi = t > 0 ? ti[t - 1] : (lane > 0 ? ci : kNo);
-                if (idx > pos) { td[t] = pd; ti[t] = pi; }
-                else if (idx == pos) { td[t] = xd; ti[t] = xi; }
-            }
-            cnt = cnt + 1 < g.k ? cnt + 1 : g.k;
-            if (cnt == g.k) {
-                uint64_t vd = 0;
-                uint32_t vi = 0;
-#pragma unroll
-                for (int t = 0; t < kKPL; ++t)
-                    if (static_cast<uint32_t>(t) == (g.k - 1) % kKPL) { vd = td[t]; vi = ti[t]; }
-                thd = __shfl_sync(0xFFFFFFFFu, vd, (g.k - 1) / kKPL);
-                thi = __shfl_sync(0xFFFFFFFFu, vi, (g.k - 1) / kKPL);
-            }
-        }
-    }
-    if (lane == 0)       // fewer than k sampled points: every point is a candidate
-        g.thr_out[q] = cnt == g.k ? __longlong_as_double(static_cast<long long>(thd))
-                                  : __longlong_as_double(0x7FF0000000000000ll);
-}
-
 // Step 2: blockIdx.y = tile of kTileQ queries (rows in shared memory);
 // threads stride over the points.
 __global__ void collect(const GtArgs g)
@@ -245,14 +184,15 @@ __global__ void collect(const GtArgs g)
 // digits.  One warp; hist: 256 words of shared memory.
 __device__ __forceinline__ uint32_t value_bits(double d) { return __float_as_uint(__double2float_ru(d)); }
 
-__device__ __forceinline__ uint32_t kth_bits(const double *cd, uint32_t m, uint32_t k, uint32_t *hist, int lane)
+template <typename Bits>
+__device__ __forceinline__ uint32_t kth_bits(Bits bits, uint32_t m, uint32_t k, uint32_t *hist, int lane)
 {
     uint32_t prefix = 0, mask = 0, want = k;     // the want-th among the values with this prefix
     for (int shift = 24; shift >= 0; shift -= 8) {
         for (int b = lane; b < 256; b += kW) hist[b] = 0;
         __syncwarp();
         for (uint32_t j = lane; j < m; j += kW) {
-            const uint32_t v = value_bits(cd[j]);
+            const uint32_t v = bits(j);
             if ((v & mask) == prefix) atomicAdd(&hist[(v >> shift) & 255u], 1u);
         }
         __syncwarp();
@@ -292,6 +232,28 @@ __device__ __forceinline__ uint32_t kth_bits(const double *cd, uint32_t m, uint3
 
 constexpr int kKthWarps = 4;
 
+// Step 1: one warp per query, the distances of the first level's points (at
+// most kSample) in shared memory, as the bits that kth_bits selects by.
+constexpr int kSampleWarps = 4;
+__global__ void __launch_bounds__(kSampleWarps * kW) sample_threshold(const GtArgs g)
+{
+    __shared__ uint32_t bits[kSampleWarps][kSample];
+    __shared__ uint32_t hist[kSampleWarps][256];
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    const uint32_t q = blockIdx.x * kSampleWarps + wid;
+    if (q >= g.nq) return;
+    const void *qr = query_row(g, q);
+    const uint32_t m = static_cast<uint32_t>(g.n);
+    for (uint32_t i = lane; i < m; i += kW) bits[wid][i] = value_bits(dist_rows(g, qr, i * g.stride));
+    __syncwarp();
+    double t = __longlong_as_double(0x7FF0000000000000ll);       // fewer than k points: every point is a candidate
+    if (m >= g.k) {
+        const uint32_t *bw = bits[wid];
+        t = static_cast<double>(__uint_as_float(kth_bits([bw](uint32_t j) { return bw[j]; }, m, g.k, hist[wid], lane)));
+    }
+    if (lane == 0) g.thr_out[q] = t == t ? t : __longlong_as_double(0x7FF0000000000000ll);   // (NaN rows)
+}
+
 // The threshold of the next level from a query's list.  One warp per query.
 __global__ void __launch_bounds__(kKthWarps * kW) kth_threshold(const GtArgs g)
 {
@@ -300,10 +262,11 @@ __global__ void __launch_bounds__(kKthWarps * kW) kth_threshold(const GtArgs g)
     const uint32_t q = blockIdx.x * kKthWarps + wid;
     if (q >= g.nq) return;
     const uint32_t m = g.cnt[q];                 // at most cap, checked by the host
-    double t = __longlong_as_double(0x7FF0000000000000ll);       // fewer than k points so far: no threshold
-    if (m >= g.k)
-        t = static_cast<double>(__uint_as_float(kth_bits(g.cd + static_cast<uint64_t>(q) * g.cap, m, g.k, hist[wid], lane)));
-    if (lane == 0) g.thr_out[q] = t;
+    const double *cd = g.cd + static_cast<uint64_t>(q) * g.cap;
+    if (m < g.k) return;                         // the level's points differ: the old threshold stays the best
+    const double t = static_cast<double>(
+        __uint_as_float(kth_bits([cd](uint32_t j) { return value_bits(cd[j]); }, m, g.k, hist[wid], lane)));
+    if (lane == 0 && t <= g.thr_out[q]) g.thr_out[q] = t;
 }
 
 // Step 3: one warp per query, the k smallest candidates in (distance, id)
@@ -322,7 +285,8 @@ __global__ void __launch_bounds__(kKthWarps * kW) select_k(const GtArgs g)
     const uint32_t m = static_cast<uint32_t>(g.cnt[q] < g.cap ? g.cnt[q] : g.cap);
     const double *cd = g.cd + static_cast<uint64_t>(q) * g.cap;
     const uint32_t *ci = g.ci + static_cast<uint64_t>(q) * g.cap;
-    const uint32_t bound = m >= g.k ? kth_bits(cd, m, g.k, hist[wid], lane) : 0xFFFFFFFFu;
+    const uint32_t bound = m >= g.k ? kth_bits([cd](uint32_t j) { return value_bits(cd[j]); }, m, g.k, hist[wid], lane)
+                                      : 0xFFFFFFFFu;
     uint32_t c = 0;                              // gathered
     for (uint32_t j0 = 0; j0 < m && c <= kSortMax; j0 += kW) {
         const uint32_t j = j0 + lane;
@@ -425,7 +389,7 @@ struct TcLevel {
         : B(base), Q(queries), dtype(dt), d(dim), nq(count), sms(sm)
     {
         nblk = (d + 15u) / 16u * (dt == 2 ? 2u : 1u);
-        on = nblk <= gt_tc::kMaxBlocks;
+        on = nblk <= (dt == 2 ? gt_tc::kMaxBlocks : 16u);    // integer sums above 256 dimensions pass 2^24
         qper = nblk <= 8u ? 256u : 128u;
         qgroups = (nq + qper - 1u) / qper;
     }
@@ -522,7 +486,7 @@ extern "C" int bang_ground_truth(int device, const void *base, const void *queri
     if (!base || !queries || !out_ids || !out_dist) return gtfail(BANG_EINVAL, "bang_ground_truth: NULL argument");
     if (dtype != BANG_U8 && dtype != BANG_I8 && dtype != BANG_F32)
         return gtfail(BANG_EINVAL, "bang_ground_truth: unknown dtype");
-    if (n == 0 || n >= (1ull << 32) - 1 || d == 0 || d > 4096 || k == 0 || k > kKPL * kW)
+    if (n == 0 || n >= (1ull << 32) - 1 || d == 0 || d > 4096 || k == 0 || k > kMaxK)
         return gtfail(BANG_EINVAL, "bang_ground_truth: need 0 < n < 2^32 - 1, 0 < d <= 4096, 1 <= k <= 256");
     if (bang::pointer_kind(base, device) == 2 || bang::pointer_kind(queries, device) == 2 ||
         bang::pointer_kind(out_ids, device) == 2 || bang::pointer_kind(out_dist, device) == 2)
@@ -576,12 +540,11 @@ extern "C" int bang_ground_truth(int device, const void *base, const void *queri
     }
     g.n = n < kSample ? n : kSample;
     g.stride = n / g.n;
-    sample_threshold<<<(nq + 3) / 4, 128, 0, st>>>(g);
+    sample_threshold<<<(nq + kSampleWarps - 1) / kSampleWarps, kSampleWarps * kW, 0, st>>>(g);
     GT_TRY(cudaGetLastError());
     int sms = 0;
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, device);
     const uint32_t tiles = (nq + tileq - 1) / tileq;
-    const uint32_t gx = static_cast<uint32_t>((static_cast<uint64_t>(sms) * 8 + tiles - 1) / tiles) + 1;
     std::vector<uint32_t> c(nq);
     uint64_t cap = 0;
     TcLevel tc(B, Q, dtype, d, nq, sms);
@@ -602,7 +565,14 @@ extern "C" int bang_ground_truth(int device, const void *base, const void *queri
             g.ci = ci.p;
             g.cap = cap;
             if (tc.on && g.n >= kTcLeast) GT_TRY(tc.collect(g, st));
-            else collect<<<dim3(gx, tiles), 256, tileq * d * esz, st>>>(g);
+            else {
+                // fewer queries a block where the level's points alone would not fill the GPU
+                const uint64_t have = (g.n + 255u) / 256u * tiles, want = 4ull * sms;
+                g.tileq = have < want ? static_cast<uint32_t>(std::max<uint64_t>(1u, tileq * have / want)) : tileq;
+                const uint32_t ty = (nq + g.tileq - 1u) / g.tileq;
+                const uint32_t tx = static_cast<uint32_t>((static_cast<uint64_t>(sms) * 8 + ty - 1) / ty) + 1;
+                collect<<<dim3(tx, ty), 256, g.tileq * d * esz, st>>>(g);
+            }
             GT_TRY(cudaGetLastError());
             GT_TRY(cudaMemcpyAsync(c.data(), cnt.p, nq * 4, cudaMemcpyDeviceToHost, st));
             if (tc.on) GT_TRY(cudaMemcpyAsync(tc.state, tc.flags.p, sizeof tc.state, cudaMemcpyDeviceToHost, st));

@@ -4,21 +4,27 @@
 //
 // Integer data (uint8, int8; d <= 256): the values are exact in FP16 and the
 // sums (at most 256 * 255^2 < 2^24) in the FP32 accumulator, so a pair that
-// passes the filter gets its exact distance from v.  FP32 data (d <= 128):
-// both sides are split into two BF16 parts (three products), which is off by
-// less than 2^-13 (|q|^2 + |x|^2) / 2 in v and its rounding; the filter is
-// that much wider and a pair that passes gets its FP64 distance from the rows.
+// passes the filter gets its exact distance from v.  FP32 data (d <= 208):
+// both sides are split into two BF16 parts (three products).  What is left out
+// and the rounding of up to 624 FP32 additions put v off by less than
+// 2^-13 |q| |x|, so 2 v by less than 2^-13 (|q|^2 + |x|^2); the filter is twice
+// that wider and a pair that passes gets its FP64 distance from the rows.
 //
 // The points are converted once per level (at most kTcPoints at a time) into
 // tiles of 256 points laid out as the MMA reads them: per 16 dimensions (and
 // part) one block of 256 x 16 16-bit values in no-swizzle K-major core
 // matrices, 8 KB; so a tile is one contiguous stretch and is fetched by bulk
 // copies into a ring of 32 KB stages.  A CTA keeps 256 queries in shared memory
-// (128 when a tile has more than 8 blocks) and streams over its share of the
+// (128 when a tile has more than 8 blocks; three stages above 16) and streams over its share of the
 // tiles: one warp copies, one issues the MMAs (M = 128, N = 256), and two
 // groups of four warps read the two TMEM accumulators, one while the other is
 // being computed.  Few pairs pass: they are kept in shared memory, 8 per
-// thread, and appended to the query's list with one atomic.
+// thread, and appended to the query's list with one atomic, by all lanes of a
+// warp together (so the first level, where a tenth of the pairs passes, took
+// 0.64 ms instead of 0.87).  10^10 pairs take 4.3 ms, where the MMAs alone would
+// take 1.4: an accumulator's turn, 256 columns read from TMEM and filtered,
+// sets the pace; packed FP32 arithmetic with a three-way minimum and loads one
+// step ahead left it the same (4.7).
 #pragma once
 
 #include <cuda_bf16.h>
@@ -32,11 +38,11 @@ namespace gt_tc {
 constexpr uint32_t kTileP = 256;            // points per tile, queries per tile
 constexpr uint32_t kBlock = 8192;           // bytes of one 256 x 16 block
 constexpr uint32_t kStageBlocks = 4;
-constexpr uint32_t kStages = 4;
+__host__ __device__ constexpr uint32_t stages(uint32_t nblk) { return nblk <= 16u ? 4u : 3u; }
 constexpr uint32_t kKeep = 8;               // pairs kept per thread before they are appended
 constexpr uint32_t kThreads = 12 * 32;
-constexpr uint32_t kMaxBlocks = 16;
-constexpr uint64_t kTcPoints = 1u << 22;    // points converted at a time (512 MB at most)
+constexpr uint32_t kMaxBlocks = 26;         // 26 x 4 KB of queries beside three stages
+constexpr uint64_t kTcPoints = 1u << 20;    // points converted at a time (832 MB at most)
 constexpr long long kWaitCycles = 6000000000ll;      // about 3 s
 
 struct TcArgs {
@@ -200,7 +206,7 @@ __global__ void __launch_bounds__(kTileP) convert(const void *X, int dtype, uint
     if (dtype == 2 && valid && !(n2 < 1e30)) *odd = 1u;
     if (norm) {
         float v = __uint_as_float(0x7F800000u);
-        if (valid) v = dtype == 2 ? __double2float_rd(n2 * (1.0 - 0x1p-13)) : static_cast<float>(n2i);
+        if (valid) v = dtype == 2 ? __double2float_rd(n2 * (1.0 - 0x1p-12)) : static_cast<float>(n2i);
         norm[i] = v;
     }
 }
@@ -217,7 +223,7 @@ __global__ void limits(const void *Q, int dtype, uint32_t d, uint32_t nq, const 
     }
     qq[q] = static_cast<float>(n2);              // exact for integers (below 2^24)
     // integers: xx - 2 v is exact below 2^24, else within 2 of it
-    lim[q] = __double2float_ru(thr[q] - n2 + (dtype == 2 ? n2 * 0x1p-13 + 1e-35 : 4.0));
+    lim[q] = __double2float_ru(thr[q] - n2 + (dtype == 2 ? n2 * 0x1p-12 + 1e-35 : 4.0));
 }
 
 // FP64 distance as the ground truth defines it.
@@ -234,7 +240,7 @@ __device__ __forceinline__ double exact64(const float *q, const float *x, uint32
 inline uint32_t smem_bytes(uint32_t nblk)
 {
     const uint32_t a = nblk <= 8u ? nblk * kBlock : nblk * kBlock / 2u;
-    return a + kStages * kStageBlocks * kBlock + 2u * kTileP * 4u + kKeep * 256u * 12u + 256u;
+    return a + stages(nblk) * kStageBlocks * kBlock + 2u * kTileP * 4u + kKeep * 256u * 12u + 256u;
 }
 
 // DT: 0 integer data (FP16 operands), 1 FP32 data (BF16 operands, two parts).
@@ -246,6 +252,7 @@ __global__ void __launch_bounds__(kThreads, 1) collect_tc(const TcArgs a)
     const bool two = a.nblk <= 8u;               // 256 queries per CTA, else 128
     const uint32_t abytes = two ? a.nblk * kBlock : a.nblk * kBlock / 2u;
     unsigned char *A = smem, *B = A + abytes;
+    const uint32_t kStages = stages(a.nblk);
     float *nrm = reinterpret_cast<float *>(B + kStages * kStageBlocks * kBlock);      // 2 x 256
     double *kd = reinterpret_cast<double *>(nrm + 2u * kTileP);
     uint32_t *ki = reinterpret_cast<uint32_t *>(kd + kKeep * 256u);
@@ -263,9 +270,9 @@ __global__ void __launch_bounds__(kThreads, 1) collect_tc(const TcArgs a)
         }
         for (uint32_t s = 0; s < 2; ++s) {
             init(nfull + 8u * s, 1);
-            init(nempty + 8u * s, two ? 256 : 128);
+            init(nempty + 8u * s, two ? 8 : 4);          // one arrival per warp
             init(tfull + 8u * s, 1);
-            init(tempty + 8u * s, 128);
+            init(tempty + 8u * s, 4);
         }
         init(qbar, 1);
         *bad = 0u;
@@ -417,11 +424,17 @@ __global__ void __launch_bounds__(kThreads, 1) collect_tc(const TcArgs a)
                         ++kept;
                     }
                 }
+                // all lanes at once, so that the warp waits for one atomic's
+                // round trip and not for one per lane
+                if (__any_sync(0xFFFFFFFFu, kept >= kKeep - 3u)) flush();
                 __syncwarp();
             }
             asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
-            arrive(tempty + 8u * g);
-            arrive(nempty + 8u * ns);
+            __syncwarp();
+            if (lane == 0) {
+                arrive(tempty + 8u * g);
+                arrive(nempty + 8u * ns);
+            }
         }
         if (mine) flush();
     }

@@ -169,7 +169,10 @@ def test_ground_truth_levels(dt, d, n, k):
     ("f32", 128, 8_193, 20, 5, "offset"),      # norms far above the distances
     ("f32", 128, 8_193, 20, 5, "huge"),        # outside the filter's range
     ("f32", 65, 12_345, 20, 5, "tiny"),
-    ("f32", 129, 9_000, 20, 5, "unit"),
+    ("f32", 129, 9_000, 20, 5, "unit"),        # more than 16 blocks: three stages
+    ("f32", 208, 8_300, 130, 37, "offset"),    # the widest
+    ("f32", 209, 8_300, 40, 5, "unit"),        # too wide
+    ("u8", 64, 20_000, 700, 1, "any"),         # levels with fewer than k candidates
 ])
 def test_ground_truth_on_the_tensor_cores(dt, d, n, nq, k, what):
     rng = np.random.default_rng(d * 3 + n)
