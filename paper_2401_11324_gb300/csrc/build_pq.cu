@@ -20,10 +20,10 @@
 // added with shared-memory atomics, a block per part of the sample; float
 // points keep the order: one warp per (subspace, centroid) looks for its points
 // in the assignments (4 bytes a lane), reads 32 points at a time and sums them.
-// 100,000 training points of u8, d = 128, M = 32: assignment 24.2 -> 0.52 ms an
+// 100,000 training points of u8, d = 128, M = 32: assignment 24.2 -> 0.45 ms an
 // iteration; update 16.6 ms with a thread per (subspace, centroid), 1.0 with the
 // warp, under 0.1 with the atomics; encoding 400,000 points 130 -> 1.6 ms.  The
-// whole call with 10 iterations: 538 -> 8.3 ms.
+// whole call with 10 iterations: 538 -> 7.6 ms.
 #include <cuda_runtime.h>
 
 #include <cstdint>
@@ -433,7 +433,11 @@ extern "C" int bang_build_pq(int device, const void *base, bang_dtype dtype, uin
     int sms = 0;
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, device);
     init_cent<<<M, 256, 0, st>>>(a, dinit.p);
-    const uint32_t bx = static_cast<uint32_t>(sms) * 4u / M + 1u;
+    // whole waves: four blocks of assign (and of update_int) fit an SM, six of
+    // encode (one block more per subspace made the 608 that fit 640: 0.52 ms
+    // an iteration instead of 0.45)
+    const uint32_t bx = static_cast<uint32_t>(sms) * 4u / M ? static_cast<uint32_t>(sms) * 4u / M : 1u;
+    const uint32_t be = static_cast<uint32_t>(sms) * 6u / M ? static_cast<uint32_t>(sms) * 6u / M : 1u;
     const uint64_t least = (ns + kIntPart - 1) / kIntPart;       // parts that keep 32-bit sums exact
     const uint32_t parts = static_cast<uint32_t>(least > bx ? least : bx);
     for (uint32_t it = 0; it < iters; ++it) {
@@ -447,7 +451,7 @@ extern "C" int bang_build_pq(int device, const void *base, bang_dtype dtype, uin
         }
     }
     to_float<<<256, 256, 0, st>>>(cent.p, 256ull * d, cb.p);
-    encode<<<dim3(bx * 4, M), 256, 0, st>>>(a);
+    encode<<<dim3(be * 3, M), 256, 0, st>>>(a);
     PQ_TRY(cudaGetLastError());
     PQ_TRY(cudaMemcpyAsync(codebook, cb.p, 256ull * d * 4, cudaMemcpyDefault, st));
     if (!codes_dev) PQ_TRY(cudaMemcpyAsync(codes, dcodes.p, n * M, cudaMemcpyDeviceToHost, st));
