@@ -43,6 +43,7 @@ constexpr int kW = 32;
 constexpr uint32_t kMaxK = 256;
 constexpr uint32_t kTileQ = 128;         // at most this many queries per CTA in pass 2
 constexpr uint32_t kSample = 1024;       // points of the first threshold
+constexpr uint64_t kQueries = 1u << 16;  // queries at a time
 constexpr uint32_t kLevel = 16;          // each further level streams over this many times as many
 
 struct GtArgs {
@@ -517,93 +518,100 @@ extern "C" int bang_ground_truth(int device, const void *base, const void *queri
         GT_TRY(cudaMemcpyAsync(dq.p, queries, static_cast<uint64_t>(nq) * d * esz, cudaMemcpyHostToDevice, st));
         Q = dq.p;
     }
-    DArr<double> thr, cd, odist;
-    DArr<uint32_t> cnt, ci, oids;
-    GT_TRY(thr.alloc(nq));
-    GT_TRY(cnt.alloc(nq));
-    GtArgs g;
-    std::memset(&g, 0, sizeof g);
-    g.base = B;
-    g.queries = Q;
-    g.dtype = dtype;
-    g.nq = nq;
-    g.d = d;
-    g.k = k;
-    g.thr_out = thr.p;
-    g.thr = thr.p;
-    g.cnt = cnt.p;
-    g.tileq = tileq;
-    {
-        const uintptr_t ab = reinterpret_cast<uintptr_t>(B), aq = reinterpret_cast<uintptr_t>(Q);
-        g.words = dtype != BANG_F32 && d % 4 == 0 && ab % 4 == 0 && aq % 4 == 0;
-        g.regrow = dtype != BANG_F32 && d % 16 == 0 && d <= 128 && ab % 16 == 0;
-    }
-    g.n = n < kSample ? n : kSample;
-    g.stride = n / g.n;
-    sample_threshold<<<(nq + kSampleWarps - 1) / kSampleWarps, kSampleWarps * kW, 0, st>>>(g);
-    GT_TRY(cudaGetLastError());
-    int sms = 0;
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, device);
-    const uint32_t tiles = (nq + tileq - 1) / tileq;
-    std::vector<uint32_t> c(nq);
-    uint64_t cap = 0;
-    TcLevel tc(B, Q, dtype, d, nq, sms);
-    GT_TRY(tc.prepare(n, st));
-    for (uint64_t seen = g.n;; seen = g.n) {
-        g.n = seen < n / kLevel ? seen * kLevel : n;     // the last level takes every point
-        g.stride = n / g.n;
-        // expected list length about k * (points now / points before); room for twice that, then the longest
-        uint64_t room = 2ull * k * ((g.n + seen - 1) / seen) + 256;
-        for (int attempt = 0;; ++attempt) {
-            if (room > cap) {
-                GT_TRY(cd.alloc(room * nq));
-                GT_TRY(ci.alloc(room * nq));
-                cap = room;
-            }
-            GT_TRY(cudaMemsetAsync(cnt.p, 0, nq * 4, st));
-            g.cd = cd.p;
-            g.ci = ci.p;
-            g.cap = cap;
-            if (tc.on && g.n >= kTcLeast) GT_TRY(tc.collect(g, st));
-            else {
-                // fewer queries a block where the level's points alone would not fill the GPU
-                const uint64_t have = (g.n + 255u) / 256u * tiles, want = 4ull * sms;
-                g.tileq = have < want ? static_cast<uint32_t>(std::max<uint64_t>(1u, tileq * have / want)) : tileq;
-                const uint32_t ty = (nq + g.tileq - 1u) / g.tileq;
-                const uint32_t tx = static_cast<uint32_t>((static_cast<uint64_t>(sms) * 8 + ty - 1) / ty) + 1;
-                collect<<<dim3(tx, ty), 256, g.tileq * d * esz, st>>>(g);
-            }
-            GT_TRY(cudaGetLastError());
-            GT_TRY(cudaMemcpyAsync(c.data(), cnt.p, nq * 4, cudaMemcpyDeviceToHost, st));
-            if (tc.on) GT_TRY(cudaMemcpyAsync(tc.state, tc.flags.p, sizeof tc.state, cudaMemcpyDeviceToHost, st));
-            GT_TRY(cudaStreamSynchronize(st));
-            if (tc.on && tc.state[1]) return gtfail(BANG_ETIMEOUT, "bang_ground_truth: a tensor-core wait gave up");
-            if (tc.on && tc.state[0]) {          // values the filter cannot bound: this level again without it
-                tc.on = false;
-                --attempt;
-                continue;
-            }
-            room = *std::max_element(c.begin(), c.end());
-            if (room <= cap) break;
-            if (attempt == 1) return gtfail(BANG_ECUDA, "bang_ground_truth: candidate lists kept growing");
-        }
-        if (g.n == n) break;
-        kth_threshold<<<(nq + kKthWarps - 1) / kKthWarps, kKthWarps * kW, 0, st>>>(g);
-        GT_TRY(cudaGetLastError());
-    }
     const bool dev_out = is_dev(out_ids);
-    if (!dev_out) {
-        GT_TRY(oids.alloc(static_cast<uint64_t>(nq) * k));
-        GT_TRY(odist.alloc(static_cast<uint64_t>(nq) * k));
+    // kQueries queries at a time: the candidate lists are sized for one block
+    for (uint64_t q0 = 0; q0 < nq; q0 += kQueries) {
+        const uint32_t m = static_cast<uint32_t>(nq - q0 < kQueries ? nq - q0 : kQueries);
+        const void *Qb = static_cast<const unsigned char *>(Q) + q0 * d * esz;
+        uint32_t *ids = out_ids + q0 * k;
+        double *dist = out_dist + q0 * k;
+        DArr<double> thr, cd, odist;
+        DArr<uint32_t> cnt, ci, oids;
+        GT_TRY(thr.alloc(m));
+        GT_TRY(cnt.alloc(m));
+        GtArgs g;
+        std::memset(&g, 0, sizeof g);
+        g.base = B;
+        g.queries = Qb;
+        g.dtype = dtype;
+        g.nq = m;
+        g.d = d;
+        g.k = k;
+        g.thr_out = thr.p;
+        g.thr = thr.p;
+        g.cnt = cnt.p;
+        g.tileq = tileq;
+        {
+            const uintptr_t ab = reinterpret_cast<uintptr_t>(B), aq = reinterpret_cast<uintptr_t>(Qb);
+            g.words = dtype != BANG_F32 && d % 4 == 0 && ab % 4 == 0 && aq % 4 == 0;
+            g.regrow = dtype != BANG_F32 && d % 16 == 0 && d <= 128 && ab % 16 == 0;
+        }
+        g.n = n < kSample ? n : kSample;
+        g.stride = n / g.n;
+        sample_threshold<<<(m + kSampleWarps - 1) / kSampleWarps, kSampleWarps * kW, 0, st>>>(g);
+        GT_TRY(cudaGetLastError());
+        int sms = 0;
+        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, device);
+        const uint32_t tiles = (m + tileq - 1) / tileq;
+        std::vector<uint32_t> c(m);
+        uint64_t cap = 0;
+        TcLevel tc(B, Qb, dtype, d, m, sms);
+        GT_TRY(tc.prepare(n, st));
+        for (uint64_t seen = g.n;; seen = g.n) {
+            g.n = seen < n / kLevel ? seen * kLevel : n;     // the last level takes every point
+            g.stride = n / g.n;
+            // expected list length about k * (points now / points before); room for twice that, then the longest
+            uint64_t room = 2ull * k * ((g.n + seen - 1) / seen) + 256;
+            for (int attempt = 0;; ++attempt) {
+                if (room > cap) {
+                    GT_TRY(cd.alloc(room * m));
+                    GT_TRY(ci.alloc(room * m));
+                    cap = room;
+                }
+                GT_TRY(cudaMemsetAsync(cnt.p, 0, m * 4, st));
+                g.cd = cd.p;
+                g.ci = ci.p;
+                g.cap = cap;
+                if (tc.on && g.n >= kTcLeast) GT_TRY(tc.collect(g, st));
+                else {
+                    // fewer queries a block where the level's points alone would not fill the GPU
+                    const uint64_t have = (g.n + 255u) / 256u * tiles, want = 4ull * sms;
+                    g.tileq = have < want ? static_cast<uint32_t>(std::max<uint64_t>(1u, tileq * have / want)) : tileq;
+                    const uint32_t ty = (m + g.tileq - 1u) / g.tileq;
+                    const uint32_t tx = static_cast<uint32_t>((static_cast<uint64_t>(sms) * 8 + ty - 1) / ty) + 1;
+                    collect<<<dim3(tx, ty), 256, g.tileq * d * esz, st>>>(g);
+                }
+                GT_TRY(cudaGetLastError());
+                GT_TRY(cudaMemcpyAsync(c.data(), cnt.p, m * 4, cudaMemcpyDeviceToHost, st));
+                if (tc.on) GT_TRY(cudaMemcpyAsync(tc.state, tc.flags.p, sizeof tc.state, cudaMemcpyDeviceToHost, st));
+                GT_TRY(cudaStreamSynchronize(st));
+                if (tc.on && tc.state[1]) return gtfail(BANG_ETIMEOUT, "bang_ground_truth: a tensor-core wait gave up");
+                if (tc.on && tc.state[0]) {          // values the filter cannot bound: this level again without it
+                    tc.on = false;
+                    --attempt;
+                    continue;
+                }
+                room = *std::max_element(c.begin(), c.end());
+                if (room <= cap) break;
+                if (attempt == 1) return gtfail(BANG_ECUDA, "bang_ground_truth: candidate lists kept growing");
+            }
+            if (g.n == n) break;
+            kth_threshold<<<(m + kKthWarps - 1) / kKthWarps, kKthWarps * kW, 0, st>>>(g);
+            GT_TRY(cudaGetLastError());
+        }
+        if (!dev_out) {
+            GT_TRY(oids.alloc(static_cast<uint64_t>(m) * k));
+            GT_TRY(odist.alloc(static_cast<uint64_t>(m) * k));
+        }
+        g.out_ids = dev_out ? ids : oids.p;
+        g.out_dist = dev_out ? dist : odist.p;
+        select_k<<<(m + kKthWarps - 1) / kKthWarps, kKthWarps * kW, 0, st>>>(g);
+        GT_TRY(cudaGetLastError());
+        if (!dev_out) {
+            GT_TRY(cudaMemcpyAsync(ids, oids.p, static_cast<uint64_t>(m) * k * 4, cudaMemcpyDeviceToHost, st));
+            GT_TRY(cudaMemcpyAsync(dist, odist.p, static_cast<uint64_t>(m) * k * 8, cudaMemcpyDeviceToHost, st));
+        }
+        GT_TRY(cudaStreamSynchronize(st));
     }
-    g.out_ids = dev_out ? out_ids : oids.p;
-    g.out_dist = dev_out ? out_dist : odist.p;
-    select_k<<<(nq + kKthWarps - 1) / kKthWarps, kKthWarps * kW, 0, st>>>(g);
-    GT_TRY(cudaGetLastError());
-    if (!dev_out) {
-        GT_TRY(cudaMemcpyAsync(out_ids, oids.p, static_cast<uint64_t>(nq) * k * 4, cudaMemcpyDeviceToHost, st));
-        GT_TRY(cudaMemcpyAsync(out_dist, odist.p, static_cast<uint64_t>(nq) * k * 8, cudaMemcpyDeviceToHost, st));
-    }
-    GT_TRY(cudaStreamSynchronize(st));
     return BANG_OK;
 }

@@ -22,9 +22,9 @@
 // thread, and appended to the query's list with one atomic, by all lanes of a
 // warp together (so the first level, where a tenth of the pairs passes, took
 // 0.64 ms instead of 0.87).  10^10 pairs take 4.3 ms, where the MMAs alone would
-// take 1.4: an accumulator's turn, 256 columns read from TMEM and filtered,
-// sets the pace; packed FP32 arithmetic with a three-way minimum and loads one
-// step ahead left it the same (4.7).
+// take 1.4: the filter's instructions set the pace (216 per 32 x 32 pairs, two
+// warps a scheduler; tensor pipe 23 %); packed FP32 arithmetic with a three-way
+// minimum and loads one step ahead left it the same (4.7).
 #pragma once
 
 #include <cuda_bf16.h>

@@ -27,9 +27,9 @@
 // iteration; the waits for rows and code rows, 40 % of it there, are gone).
 // So where the entry after u* is ready too, both are expanded in one step (a
 // quarter to a third of the steps); an expander takes about 3,000 cycles, hence
-// three.  10,000 u8 queries, 1M points, L = 224, FP32 table, HBM: 7.04 -> 5.10 ms;
-// 3,000 float queries, d = 96, M = 48, L = 128: 4.22 -> 2.53 ms; one query at
-// L = 64: 218 -> 157 us (169 -> 125 on another day).
+// three.  10,000 u8 queries, 1M points, L = 224, FP32 table, HBM: 7.02 -> 5.06 ms;
+// 3,000 float queries, d = 96, M = 48, L = 128: 4.33 -> 2.57 ms; one query at
+// L = 64: 156 -> 112 us.
 //
 // Slots are handed over through two mbarriers each (request, result); every
 // wait is bounded, and a wait that gave up ends the query with status 3.

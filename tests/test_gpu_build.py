@@ -173,6 +173,7 @@ def test_ground_truth_levels(dt, d, n, k):
     ("f32", 208, 8_300, 130, 37, "offset"),    # the widest
     ("f32", 209, 8_300, 40, 5, "unit"),        # too wide
     ("u8", 64, 20_000, 700, 1, "any"),         # levels with fewer than k candidates
+    ("i8", 8, 8_200, 66_000, 3, "any"),        # more queries than one block of them
 ])
 def test_ground_truth_on_the_tensor_cores(dt, d, n, nq, k, what):
     rng = np.random.default_rng(d * 3 + n)
