@@ -22,7 +22,7 @@
 // d = 128, 1M points, k = 100).  Over 1,024, with the distances in shared memory
 // and a radix selection, it takes 1.2.  The streamed levels are a contraction:
 // with a point per thread (vabsdiff4 + dp4a) they took 73 ms, on the tensor
-// cores 7.4; the sorted selection took 3.9 ms one neighbour after the other, 0.1
+// cores 6.1; the sorted selection took 3.9 ms one neighbour after the other, 0.1
 // gathered and sorted.
 #include <cuda_runtime.h>
 

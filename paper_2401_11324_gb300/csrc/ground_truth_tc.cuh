@@ -17,14 +17,15 @@
 // copies into a ring of 32 KB stages.  A CTA keeps 256 queries in shared memory
 // (128 when a tile has more than 8 blocks; three stages above 16) and streams over its share of the
 // tiles: one warp copies, one issues the MMAs (M = 128, N = 256), and two
-// groups of four warps read the two TMEM accumulators, one while the other is
-// being computed.  Few pairs pass: they are kept in shared memory, 8 per
-// thread, and appended to the query's list with one atomic, by all lanes of a
-// warp together (so the first level, where a tenth of the pairs passes, took
-// 0.64 ms instead of 0.87).  10^10 pairs take 4.3 ms, where the MMAs alone would
-// take 1.4: the filter's instructions set the pace (216 per 32 x 32 pairs, two
-// warps a scheduler; tensor pipe 23 %); packed FP32 arithmetic with a three-way
-// minimum and loads one step ahead left it the same (4.7).
+// groups of eight warps read the two TMEM accumulators, half the columns each,
+// one accumulator while the other is being computed.  Few pairs pass: they are
+// kept in shared memory, 4 per thread, and appended to the query's list with
+// one atomic, by all lanes of a warp together (so the first level, where a tenth
+// of the pairs passes, took 0.64 ms instead of 0.87).  The filter's instructions
+// set the pace (216 per 32 x 32 pairs; 10^10 pairs take the MMAs alone 1.4 ms):
+// with four warps a group, two a scheduler, the three levels of 10,000 queries
+// over 1M points took 7.5 ms (tensor pipe 23 %), with eight 6.1; packed FP32
+// arithmetic with a three-way minimum and loads one step ahead changed nothing.
 #pragma once
 
 #include <cuda_bf16.h>
@@ -39,8 +40,9 @@ constexpr uint32_t kTileP = 256;            // points per tile, queries per tile
 constexpr uint32_t kBlock = 8192;           // bytes of one 256 x 16 block
 constexpr uint32_t kStageBlocks = 4;
 __host__ __device__ constexpr uint32_t stages(uint32_t nblk) { return nblk <= 16u ? 4u : 3u; }
-constexpr uint32_t kKeep = 8;               // pairs kept per thread before they are appended
-constexpr uint32_t kThreads = 12 * 32;
+constexpr uint32_t kKeep = 4;               // pairs kept per thread before they are appended
+constexpr uint32_t kFilter = 512;           // filtering threads: two per accumulator row
+constexpr uint32_t kThreads = 128 + kFilter;
 constexpr uint32_t kMaxBlocks = 26;         // 26 x 4 KB of queries beside three stages
 constexpr uint64_t kTcPoints = 1u << 20;    // points converted at a time (832 MB at most)
 constexpr long long kWaitCycles = 6000000000ll;      // about 3 s
@@ -240,7 +242,7 @@ __device__ __forceinline__ double exact64(const float *q, const float *x, uint32
 inline uint32_t smem_bytes(uint32_t nblk)
 {
     const uint32_t a = nblk <= 8u ? nblk * kBlock : nblk * kBlock / 2u;
-    return a + stages(nblk) * kStageBlocks * kBlock + 2u * kTileP * 4u + kKeep * 256u * 12u + 256u;
+    return a + stages(nblk) * kStageBlocks * kBlock + 2u * kTileP * 4u + kKeep * kFilter * 12u + 256u;
 }
 
 // DT: 0 integer data (FP16 operands), 1 FP32 data (BF16 operands, two parts).
@@ -255,8 +257,8 @@ __global__ void __launch_bounds__(kThreads, 1) collect_tc(const TcArgs a)
     const uint32_t kStages = stages(a.nblk);
     float *nrm = reinterpret_cast<float *>(B + kStages * kStageBlocks * kBlock);      // 2 x 256
     double *kd = reinterpret_cast<double *>(nrm + 2u * kTileP);
-    uint32_t *ki = reinterpret_cast<uint32_t *>(kd + kKeep * 256u);
-    uint64_t *bars = reinterpret_cast<uint64_t *>(ki + kKeep * 256u);
+    uint32_t *ki = reinterpret_cast<uint32_t *>(kd + kKeep * kFilter);
+    uint64_t *bars = reinterpret_cast<uint64_t *>(ki + kKeep * kFilter);
     const uint32_t b0 = saddr(bars);
     // full / empty stage, full / empty norms, full / empty accumulator, queries
     const uint32_t full = b0, empty = b0 + 32u, nfull = b0 + 64u, nempty = b0 + 80u, tfull = b0 + 96u,
@@ -270,9 +272,9 @@ __global__ void __launch_bounds__(kThreads, 1) collect_tc(const TcArgs a)
         }
         for (uint32_t s = 0; s < 2; ++s) {
             init(nfull + 8u * s, 1);
-            init(nempty + 8u * s, two ? 8 : 4);          // one arrival per warp
+            init(nempty + 8u * s, two ? 16 : 8);          // one arrival per warp
             init(tfull + 8u * s, 1);
-            init(tempty + 8u * s, 4);
+            init(tempty + 8u * s, 8);
         }
         init(qbar, 1);
         *bad = 0u;
@@ -364,8 +366,8 @@ __global__ void __launch_bounds__(kThreads, 1) collect_tc(const TcArgs a)
             }
         }
     } else if (warp >= 4) {
-        // ---- filter: this thread's query against the tile's 256 points
-        const uint32_t g = (warp - 4u) >> 2, r = (warp & 3u) * 32u + lane, me = tid - 128u;
+        // ---- filter: this thread's query against half of the tile's points
+        const uint32_t g = (warp - 4u) >> 3, half = ((warp - 4u) >> 2) & 1u, r = (warp & 3u) * 32u + lane, me = tid - 128u;
         const uint32_t q = q0 + (two ? g * 128u : 0u) + r;
         const bool mine = q < a.nq;
         const float lim = mine ? a.lim[q] : __uint_as_float(0xFF800000u);
@@ -377,8 +379,8 @@ __global__ void __launch_bounds__(kThreads, 1) collect_tc(const TcArgs a)
             const uint32_t at = atomicAdd(a.cnt + q, kept);
             for (uint32_t i = 0; i < kept; ++i)
                 if (at + i < a.cap) {
-                    a.cd[static_cast<uint64_t>(q) * a.cap + at + i] = kd[i * 256u + me];
-                    a.ci[static_cast<uint64_t>(q) * a.cap + at + i] = ki[i * 256u + me];
+                    a.cd[static_cast<uint64_t>(q) * a.cap + at + i] = kd[i * kFilter + me];
+                    a.ci[static_cast<uint64_t>(q) * a.cap + at + i] = ki[i * kFilter + me];
                 }
             kept = 0;
         };
@@ -388,7 +390,7 @@ __global__ void __launch_bounds__(kThreads, 1) collect_tc(const TcArgs a)
             if (!__all_sync(0xFFFFFFFFu, ok)) break;
             asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
             const float4 *xn = reinterpret_cast<const float4 *>(nrm + ns * kTileP);
-            for (uint32_t c0 = 0; c0 < kTileP; c0 += 32) {
+            for (uint32_t c0 = half * (kTileP / 2u); c0 < (half + 1u) * (kTileP / 2u); c0 += 32) {
                 float v[32];
                 ld32(tmem + g * 256u + (((warp & 3u) * 32u) << 16) + c0, v);
                 uint32_t pass = 0;
@@ -419,14 +421,14 @@ __global__ void __launch_bounds__(kThreads, 1) collect_tc(const TcArgs a)
                     }
                     if (dist <= thr) {
                         if (kept == kKeep) flush();
-                        kd[kept * 256u + me] = dist;
-                        ki[kept * 256u + me] = static_cast<uint32_t>(id);
+                        kd[kept * kFilter + me] = dist;
+                        ki[kept * kFilter + me] = static_cast<uint32_t>(id);
                         ++kept;
                     }
                 }
                 // all lanes at once, so that the warp waits for one atomic's
                 // round trip and not for one per lane
-                if (__any_sync(0xFFFFFFFFu, kept >= kKeep - 3u)) flush();
+                if (__any_sync(0xFFFFFFFFu, kept >= kKeep - 1u)) flush();
                 __syncwarp();
             }
             asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
