@@ -493,8 +493,11 @@ __global__ void __maxnreg__(team_regs(DCH, MODE)) team_kernel(const SearchArgs a
                 // unless one of u*'s new neighbours is nearer.  When its slot
                 // is ready too and both nodes' neighbours fit the warp, they
                 // are filtered together, u*'s first.
-                bool pair = lkey != ~0ull && s2 < nexp && both3 && iters + 1u < iter_cap &&
-                            team_test(result(s2), (phase >> s2) & 1u);
+                // (Each lane asks for itself while the expander may arrive at
+                // any moment: the vote makes one answer of it, which the
+                // branches and votes below need.)
+                bool pair = lkey != ~0ull && s2 < nexp && both3 && iters + 1u < iter_cap;
+                if (pair) pair = __all_sync(0xFFFFFFFFu, team_test(result(s2), (phase >> s2) & 1u)) != 0;
                 const uint32_t m = head[3u * se + 1u], xd = head[3u * se + 2u];
                 uint32_t m2 = 0, xd2 = 0;
                 if (pair) {

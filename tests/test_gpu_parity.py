@@ -897,3 +897,26 @@ def test_final_worklist_rerank_other_types_and_batched(u8small):
             sel = np.where((k == kk) & (L == LL))[0]
             o = oracle_search(u8small, Q[sel], int(kk), int(LL), rerank_list=True)
             assert (ids[sel, :kk] == o["ids"]).all()
+
+
+@pytest.mark.parametrize("mode", [0, 1])
+def test_team_search_repeats_itself(u8small, mode):
+    # the control warp takes two expansions at once when the second one's
+    # result is there already, which depends on timing: whenever it arrives,
+    # every run gives the same visits and results
+    Q = np.resize(u8small["queries"], (900, u8small["queries"].shape[1]))
+    w = u8small
+    ix = bang.Index(w["base"], w["codebook"], w["codes"], w["adj"], w["medoid"], w["M"])
+    q = torch.from_numpy(np.ascontiguousarray(Q)).cuda()
+    ref = None
+    for rep in range(60):
+        nq = (900, 37, 450)[rep % 3]
+        ids = torch.empty((nq, 10), dtype=torch.int32, device="cuda")
+        dist = torch.empty((nq, 10), dtype=torch.float32, device="cuda")
+        iters = torch.empty(nq, dtype=torch.int32, device="cuda")
+        ix.search(q[:nq], 10, 96, ids, dist, bang.make_params(mode=mode, out_iters=iters))
+        if ref is None:
+            ref = (ids, dist, iters)
+        for x, y in zip((ids, dist, iters), ref):
+            assert torch.equal(x, y[:nq])
+    ix.close()
