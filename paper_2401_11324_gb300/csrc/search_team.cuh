@@ -820,6 +820,7 @@ inline uint32_t team_expanders(const SearchArgs &a, int mode, int sms)
 {
     const uint32_t smem = ((TeamLayout(a.M, a.log2z, a.L, a.k, a.d, a.R, mode, 2).total + 127u) & ~127u) + 1024u;
     const uint32_t fit = 228u * 1024u / smem, share = (a.nq + static_cast<uint32_t>(sms) - 1u) / static_cast<uint32_t>(sms);
+    if (fit == 0u) return 0u;      // two slots are more shared memory than a CTA may have: the one-warp form's fits
     // launches that overlap (the server's) fill the SMs together, and all take
     // the same form: 24 requests, BF16 table, L up to 256 (c = 7), against one
     // warp per query: two expanders 1.02 times as fast, three 1.06; the form

@@ -141,3 +141,26 @@ def test_admission_by_device_memory(index):
     ids, _, _ = small.wait(t, timeout_ms=60_000)
     assert (ids != bang.BANG_NONE).any()
     small.stop()
+
+
+@pytest.mark.parametrize("Lmax", [64, 80, 96])
+def test_server_where_only_the_one_warp_form_fits(Lmax):
+    # a 2^20-bit filter and 96 subspaces of FP32 entries take 131,072 + 98,304
+    # of the 232,448 bytes of shared memory a query may have: one warp's
+    # search fits beside them, the expander warps' slots do not (two of them do
+    # at L = 64)
+    w = cases.clustered(n=5_000, nq=60, ncomp=4, dtype="f32", d=96, M=96, R=32, centre="uniform255")
+    ix = bang.Index(w["base"], w["codebook"], w["codes"], w["adj"], w["medoid"], 96)
+    k = np.full(60, 10, np.uint32)
+    L = np.linspace(10, Lmax, 60).astype(np.uint32)
+    want = np.zeros((60, 10), np.uint32), np.zeros((60, 10), np.float32)
+    ix.search_batched(w["queries"], k, L, 10, Lmax, *want, bang.make_params(bloom_log2=20))
+    srv = bang.Server(ix, 10, Lmax, max_batch=32, streams=2, bloom_log2=20)
+    tickets = [srv.submit(w["queries"][i:i + 20], k[i:i + 20], L[i:i + 20]) for i in (0, 20, 40)]
+    try:
+        for i, t in zip((0, 20, 40), tickets):
+            ids, dist, _ = srv.wait(t, 20_000)
+            assert (ids == want[0][i:i + 20]).all() and (dist == want[1][i:i + 20]).all()
+    finally:
+        srv.stop()
+        ix.close()
