@@ -370,8 +370,10 @@ cudaError_t launch_tc_tables(const TcTableArgs &args, int dtype, cudaStream_t st
     const uint32_t smem = smem_for(a.nbmax, dtype);
     const dim3 grid((a.nq + kTile - 1) / kTile, (a.M + kSubPerCta - 1) / kSubPerCta);
     cudaError_t e;
+    // the limit belongs to the kernel, not to this call: every thread sets the
+    // same one, or one thread's layout would refuse another's launch
 #define BANG_TC_LAUNCH(DT)                                                                          \
-    e = cudaFuncSetAttribute(adc_table_tc_kernel<DT>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem); \
+    e = cudaFuncSetAttribute(adc_table_tc_kernel<DT>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024); \
     if (e != cudaSuccess) return e;                                                                 \
     adc_table_tc_kernel<DT><<<grid, 128, smem, st>>>(a)
     if (dtype == 0) { BANG_TC_LAUNCH(0); }

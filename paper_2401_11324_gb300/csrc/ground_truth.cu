@@ -410,9 +410,11 @@ struct TcLevel {
         if ((e = qq.alloc(nq)) != cudaSuccess) return e;
         if ((e = flags.alloc(2)) != cudaSuccess) return e;
         if ((e = cudaMemsetAsync(flags.p, 0, 8, st)) != cudaSuccess) return e;
-        const int smem = static_cast<int>(gt_tc::smem_bytes(nblk));
-        e = dtype == 2 ? cudaFuncSetAttribute(gt_tc::collect_tc<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem)
-                       : cudaFuncSetAttribute(gt_tc::collect_tc<0>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+        // the limit belongs to the kernel and outlasts this call: the same for every
+        // thread, as others launch with theirs between this call's levels
+        constexpr int kMost = 227 * 1024;
+        e = dtype == 2 ? cudaFuncSetAttribute(gt_tc::collect_tc<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, kMost)
+                       : cudaFuncSetAttribute(gt_tc::collect_tc<0>, cudaFuncAttributeMaxDynamicSharedMemorySize, kMost);
         if (e != cudaSuccess) return e;
         gt_tc::convert<<<qt, gt_tc::kTileP, 0, st>>>(Q, dtype, d, nblk, 0, nq, 1, qtiles.p, nullptr, flags.p);
         return cudaGetLastError();
