@@ -398,7 +398,8 @@ int bang_build_cluster_graph(int device, const void *base, bang_dtype dtype, uin
  * Device memory: about n*ell*(R*4 + d*elem rounded to 16, then to 32 bytes
  * per record) plus per-round scratch (about 40*R bytes per member of the
  * largest round, and 8 bytes per candidate of the longest reverse-edge
- * lists).  Blocks until done. */
+ * lists).  Blocks until done.  BANG_ETIMEOUT if a bounded wait inside one of
+ * its searches gave up. */
 int bang_build_shard_graph(int device, const void *base, bang_dtype dtype, uint64_t n, uint32_t d,
                            const float *centres, uint32_t S, uint32_t ell, uint32_t R, uint32_t Lb,
                            float alpha, float batch_frac, uint32_t log2z, uint32_t iter_cap,
@@ -530,7 +531,9 @@ int bang_server_submit(bang_server *s, const void *queries, uint32_t nq, const u
 /* Wait up to timeout_ms (negative: no limit) for a request, copy its results
  * (nq*k_max ids and distances, rows padded as bang_search_batched) to host
  * memory and release the ticket; *latency_ms = submit to results in host
- * memory.  BANG_ETIMEOUT leaves the ticket valid. */
+ * memory.  BANG_ETIMEOUT leaves the ticket valid.  BANG_ECUDA: the batch's
+ * launch failed, or a bounded wait inside its search gave up (status 3 of
+ * bang_search_params.out_status), so that no result is returned. */
 int bang_server_wait(bang_server *s, uint64_t ticket, int32_t timeout_ms, uint32_t *out_ids,
                      float *out_dist, double *latency_ms);
 /* Finish queued and running requests, then free the server. */

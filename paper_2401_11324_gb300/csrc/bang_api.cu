@@ -707,7 +707,7 @@ namespace {
 int search_impl(bang_index *ix, const void *queries, uint32_t nq, uint32_t k, uint32_t L,
                 const uint32_t *k_arr, const uint32_t *L_arr, bool persistent,
                 const bang_search_params *params, uint32_t *out_ids, float *out_dist, void *stream,
-                bool overlapped = false)
+                const bang::SearchForm &form = bang::SearchForm())
 {
     if (!ix) return fail(BANG_EINVAL, "bang_search: index is NULL");
     if (!ix->have_pq || !ix->have_graph || !ix->have_vectors)
@@ -867,7 +867,13 @@ int search_impl(bang_index *ix, const void *queries, uint32_t nq, uint32_t k, ui
     a.phase_cycles = static_cast<unsigned long long *>(dptr(7));
     a.carveout = p.smem_carveout;
     a.ntab = ntab;
-    a.overlapped = overlapped ? 1u : 0u;
+    a.overlapped = form.overlapped ? 1u : 0u;
+    a.form = form.form;
+    a.form_out = form.form_out;
+    a.wait_cycles = form.wait_cycles;
+    a.gave_up = form.gave_up;
+    a.mute = form.mute;
+    if (form.form_out) *form.form_out = 1u;
     if (p.rerank != 0) {       // staged re-rank: lists sized by the iteration cap (or L)
         uint64_t cap = p.iter_cap ? p.iter_cap : 8ull * L + 64ull;
         if (cap < L) cap = L;
@@ -928,13 +934,25 @@ int search_impl(bang_index *ix, const void *queries, uint32_t nq, uint32_t k, ui
 
 int bang::search_batched(bang_index *ix, const void *queries, uint32_t nq, const uint32_t *k_per_q,
                          const uint32_t *L_per_q, uint32_t k_max, uint32_t L_max, const bang_search_params *params,
-                         uint32_t *out_ids, float *out_dist, void *stream, bool overlapped)
+                         uint32_t *out_ids, float *out_dist, void *stream, const SearchForm &form)
 {
-    return search_impl(ix, queries, nq, k_max, L_max, k_per_q, L_per_q, true, params, out_ids, out_dist, stream,
-                       overlapped);
+    return search_impl(ix, queries, nq, k_max, L_max, k_per_q, L_per_q, true, params, out_ids, out_dist, stream, form);
 }
 
 extern "C" {
+
+int bang_internal_search(bang_index *ix, const void *queries, uint32_t nq, const uint32_t *k_per_q,
+                         const uint32_t *L_per_q, uint32_t k, uint32_t L, const bang_search_params *params,
+                         uint32_t *out_ids, float *out_dist, void *stream, uint32_t form, long long wait_cycles,
+                         uint32_t mute, uint32_t *form_out)
+{
+    bang::SearchForm f;
+    f.form = form;
+    f.form_out = form_out;
+    f.wait_cycles = wait_cycles;
+    f.mute = mute;
+    return search_impl(ix, queries, nq, k, L, k_per_q, L_per_q, k_per_q != nullptr, params, out_ids, out_dist, stream, f);
+}
 
 int bang_search(bang_index *ix, const void *queries, uint32_t nq, uint32_t k, uint32_t L,
                 const bang_search_params *params, uint32_t *out_ids, float *out_dist,

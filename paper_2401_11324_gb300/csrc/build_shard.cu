@@ -903,12 +903,11 @@ cudaError_t run_lists(LArgs a, BigScratch &bs, cudaStream_t st)
                         : launch_big<2>(a, bs.defer.p, nd, bs.off.p, bs.region.p, smem, st);
 }
 
-}  // namespace
-
-extern "C" int bang_build_shard_graph(int device, const void *base, bang_dtype dtype, uint64_t n, uint32_t d,
-                                      const float *centres, uint32_t S, uint32_t ell, uint32_t R, uint32_t Lb,
-                                      float alpha, float batch_frac, uint32_t log2z, uint32_t iter_cap,
-                                      uint32_t *adj, uint32_t *shard_of, void *stream)
+// bang_build_shard_graph; the searches' form, the limit of their waits and a
+// silent query as SearchArgs has them.
+int build(int device, const void *base, bang_dtype dtype, uint64_t n, uint32_t d, const float *centres, uint32_t S,
+          uint32_t ell, uint32_t R, uint32_t Lb, float alpha, float batch_frac, uint32_t log2z, uint32_t iter_cap,
+          uint32_t *adj, uint32_t *shard_of, void *stream, uint32_t form, long long wait_cycles, uint32_t mute)
 {
     if (!base || !centres || !adj) return sfail(BANG_EINVAL, "bang_build_shard_graph: NULL argument");
     if (dtype != BANG_U8 && dtype != BANG_I8 && dtype != BANG_F32)
@@ -1056,7 +1055,8 @@ extern "C" int bang_build_shard_graph(int device, const void *base, bang_dtype d
     SG_TRY(fill.alloc(std::min<uint64_t>(nv, static_cast<uint64_t>(max_round) * R)));
     SG_TRY(toff.alloc(std::min<uint64_t>(nv, static_cast<uint64_t>(max_round) * R)));
     SG_TRY(in_src.alloc(static_cast<uint64_t>(max_round) * R));
-    SG_TRY(ntouched.alloc(1));
+    SG_TRY(ntouched.alloc(2));                     // touched nodes of a round; a search's wait gave up
+    SG_TRY(cudaMemsetAsync(ntouched.p, 0, 8, st));
     SG_TRY(bs.ndefer.alloc(1));
     SG_TRY(cudaMemsetAsync(cntv.p, 0, sizeof(uint32_t) * nv, st));
 
@@ -1073,6 +1073,10 @@ extern "C" int bang_build_shard_graph(int device, const void *base, bang_dtype d
     sa.vec_ok = d % 4 == 0 ? 1u : 0u;              // 4-element loads stay inside aligned rows
     sa.vecb_ok = d % 4 == 0 ? 1u : 0u;
     sa.trace_cap = iter_cap;
+    sa.form = form;
+    sa.wait_cycles = wait_cycles;
+    sa.gave_up = ntouched.p + 1;
+    sa.mute = mute;
     const bang::SmemLayout lay(1, log2z, Lb, 1, d, R, bang::kModeExact);
 
     LArgs la;
@@ -1141,9 +1145,11 @@ extern "C" int bang_build_shard_graph(int device, const void *base, bang_dtype d
             rev_count<<<blocks(static_cast<uint64_t>(rn) * R, 256), 256, 0, st>>>(staging.p, rn, R, cntv.p, tpos.p,
                                                                                touched.p, ntouched.p);
             SG_TRY(cudaGetLastError());
-            uint32_t nt = 0;
-            SG_TRY(cudaMemcpyAsync(&nt, ntouched.p, 4, cudaMemcpyDeviceToHost, st));
+            uint32_t state[2] = {0u, 0u};
+            SG_TRY(cudaMemcpyAsync(state, ntouched.p, sizeof state, cudaMemcpyDeviceToHost, st));
             SG_TRY(cudaStreamSynchronize(st));
+            if (state[1]) return sfail(BANG_ETIMEOUT, "bang_build_shard_graph: a bounded wait inside a search gave up");
+            const uint32_t nt = state[0];
             if (nt == 0) continue;
             rev_counts_of_touched<<<blocks(nt, 256), 256, 0, st>>>(touched.p, nt, cntv.p, tcnt.p);
             SG_TRY(scan_counts(tcnt.p, nt, toff.p, bsum, st));
@@ -1190,4 +1196,25 @@ extern "C" int bang_build_shard_graph(int device, const void *base, bang_dtype d
     }
     SG_TRY(cudaStreamSynchronize(st));
     return BANG_OK;
+}
+
+}  // namespace
+
+extern "C" int bang_build_shard_graph(int device, const void *base, bang_dtype dtype, uint64_t n, uint32_t d,
+                                      const float *centres, uint32_t S, uint32_t ell, uint32_t R, uint32_t Lb,
+                                      float alpha, float batch_frac, uint32_t log2z, uint32_t iter_cap,
+                                      uint32_t *adj, uint32_t *shard_of, void *stream)
+{
+    return build(device, base, dtype, n, d, centres, S, ell, R, Lb, alpha, batch_frac, log2z, iter_cap, adj, shard_of,
+                 stream, 0, 0, 0);
+}
+
+extern "C" int bang_internal_build_shard_graph(int device, const void *base, int dtype, uint64_t n, uint32_t d,
+                                               const float *centres, uint32_t S, uint32_t ell, uint32_t R,
+                                               uint32_t Lb, float alpha, float batch_frac, uint32_t log2z,
+                                               uint32_t iter_cap, uint32_t *adj, uint32_t *shard_of, void *stream,
+                                               uint32_t form, long long wait_cycles, uint32_t mute)
+{
+    return build(device, base, static_cast<bang_dtype>(dtype), n, d, centres, S, ell, R, Lb, alpha, batch_frac, log2z,
+                 iter_cap, adj, shard_of, stream, form, wait_cycles, mute);
 }

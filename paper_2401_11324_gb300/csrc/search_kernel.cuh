@@ -111,6 +111,12 @@ struct SearchArgs {
     uint32_t cand_list;       // 1: the candidates are the final worklist instead (cand_cap >= L)
     uint32_t carveout;        // preferred shared-memory share of L1 in percent (0: the CUDA driver's choice)
     uint32_t overlapped;      // other launches share the GPU (chooses the form of the search only)
+    uint32_t form;            // 0: chosen at the launch; 1: one warp a query; 1 + E: a team with E expanders
+    uint32_t *form_out;       // host memory or null: the form launched, counted like `form`
+    // Team form: what becomes of its bounded waits (search_team.cuh).
+    long long wait_cycles;    // SM cycles until one gives up (0: kTeamWaitCycles)
+    uint32_t *gave_up;        // device-accessible or null: set to 1 when one did
+    uint32_t mute;            // 1 + the query whose first expander answers nothing (0: none), for tests
     uint32_t ntab;            // kModeF32Lazy: subspaces (the first ones) whose entries stay in a table
 };
 

@@ -32,7 +32,10 @@
 // L = 64: 156 -> 112 us.
 //
 // Slots are handed over through two mbarriers each (request, result); every
-// wait is bounded, and a wait that gave up ends the query with status 3.
+// wait is bounded.  A control warp whose wait gave up ends the query with
+// status 3 and sets SearchArgs::gave_up.  Whichever side gave up, the two may
+// then count a slot's phases differently, so the CTA starts its next query with
+// new barriers.
 #pragma once
 
 #include "search_kernel.cuh"
@@ -61,7 +64,7 @@ struct TeamLayout {
         slot_bytes = rw * (log2z <= 16u ? 12u : 16u);     // ids, distances, filter positions
         off_slot = o;   o += E * slot_bytes;
         off_qw = o;     o += mode == kModeExact ? 128u : 0u;   // the query's bytes (integer vectors, d <= 128)
-        off_head = o;   o += SmemLayout::up16(E * 12u + 4u);   // node, count, exact distance; query ticket
+        off_head = o;   o += SmemLayout::up16(E * 12u + 8u);   // node, count, exact distance; query ticket; a wait gave up
         off_bar = o;    o += SmemLayout::up16(E * 16u);
         // table-build scratch, dead before the first slot is used
         const uint32_t sq = SmemLayout::up16(mode != kModeExact ? d * 4u : 0u),
@@ -85,6 +88,10 @@ __device__ __forceinline__ void team_bar_init(uint32_t bar)
 {
     asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;\n" ::"r"(bar) : "memory");
 }
+__device__ __forceinline__ void team_bar_inval(uint32_t bar)
+{
+    asm volatile("mbarrier.inval.shared::cta.b64 [%0];\n" ::"r"(bar) : "memory");
+}
 __device__ __forceinline__ void team_arrive(uint32_t bar)
 {
     asm volatile("{\n\t.reg .b64 t;\n\tmbarrier.arrive.release.cta.shared::cta.b64 t, [%0];\n\t}\n" ::"r"(bar)
@@ -102,8 +109,8 @@ __device__ __forceinline__ bool team_test(uint32_t bar, uint32_t parity)
         : "memory");
     return ok != 0u;
 }
-// Whole warp; false when the wait gave up.
-__device__ __forceinline__ bool team_wait(uint32_t bar, uint32_t parity)
+// Whole warp; false when the wait gave up, after about `limit` cycles.
+__device__ __forceinline__ bool team_wait(uint32_t bar, uint32_t parity, long long limit)
 {
     uint32_t ok = 0;
     long long began = 0;
@@ -117,7 +124,7 @@ __device__ __forceinline__ bool team_wait(uint32_t bar, uint32_t parity)
             : "memory");
         if (ok) break;
         if (i == 0) began = clock64();
-        else if (clock64() - began > kTeamWaitCycles) break;
+        else if (clock64() - began > limit) break;
     }
     return __all_sync(0xFFFFFFFFu, ok != 0u) != 0;
 }
@@ -281,7 +288,8 @@ __global__ void __maxnreg__(team_regs(DCH, MODE)) team_kernel(const SearchArgs a
     uint64_t *Ck = reinterpret_cast<uint64_t *>(smem + lay.off_Ck);
     uint32_t *qw = reinterpret_cast<uint32_t *>(smem + lay.off_qw);
     volatile uint32_t *head = reinterpret_cast<volatile uint32_t *>(smem + lay.off_head);   // 3 words per slot
-    volatile uint32_t *ticket = head + 3u * nexp;
+    volatile uint32_t *ticket = head + 3u * nexp, *gave_up = ticket + 1;
+    const long long limit = a.wait_cycles ? a.wait_cycles : kTeamWaitCycles;
     const uint32_t bar0 = team_smem_addr(smem + lay.off_bar);   // slot e: request at +16e, result at +16e+8
     float *qv = reinterpret_cast<float *>(smem + lay.off_q);
     uint32_t *offs = reinterpret_cast<uint32_t *>(smem + lay.off_offs);
@@ -297,6 +305,7 @@ __global__ void __maxnreg__(team_regs(DCH, MODE)) team_kernel(const SearchArgs a
     if (threadIdx.x == 0) {
         for (uint32_t i = 0; i < 2u * nexp; ++i) team_bar_init(bar0 + 8u * i);
         asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
+        *gave_up = 0u;
     }
     __syncthreads();
 
@@ -364,7 +373,10 @@ __global__ void __maxnreg__(team_regs(DCH, MODE)) team_kernel(const SearchArgs a
             uint32_t *db = ids + rw;
             const uint32_t req = bar0 + 16u * e;
             for (;;) {
-                if (!team_wait(req, phase)) break;
+                if (!team_wait(req, phase, limit) || (e == 0u && q + 1u == a.mute)) {
+                    if (lane == 0) *gave_up = 1u;
+                    break;
+                }
                 phase ^= 1u;
                 const uint32_t u = head[3u * e];
                 if (u == kNone) break;                   // the query is done
@@ -485,7 +497,7 @@ __global__ void __maxnreg__(team_regs(DCH, MODE)) team_kernel(const SearchArgs a
                 // (one bit at most: the leading-zero count is half of __ffs)
                 const uint32_t se = 31u - __clz(__ballot_sync(0xFFFFFFFFu, sid == u));
                 const uint32_t s2 = 31u - __clz(__ballot_sync(0xFFFFFFFFu, sid == u2));     // ~0: in no slot
-                if (!team_wait(result(se), (phase >> se) & 1u)) {
+                if (!team_wait(result(se), (phase >> se) & 1u, limit)) {
                     status = 3;
                     break;
                 }
@@ -757,7 +769,7 @@ __global__ void __maxnreg__(team_regs(DCH, MODE)) team_kernel(const SearchArgs a
             // ---- end of the query: the expanders finish and stop
             for (uint32_t e = 0; e < nexp; ++e) {
                 if (__shfl_sync(0xFFFFFFFFu, sid, static_cast<int>(e)) != kNone) {
-                    if (!team_wait(result(e), (phase >> e) & 1u)) status = 3;
+                    if (!team_wait(result(e), (phase >> e) & 1u, limit)) status = 3;
                     phase ^= 1u << e;
                 }
                 if (static_cast<uint32_t>(lane) == e) {
@@ -794,9 +806,26 @@ __global__ void __maxnreg__(team_regs(DCH, MODE)) team_kernel(const SearchArgs a
                 if (a.out_iters) a.out_iters[q] = iters;
                 if (a.out_status) a.out_status[q] = status;
                 if (a.out_ndist) a.out_ndist[q] = ndist;
+                if (status == 3) {
+                    *gave_up = 1u;
+                    if (a.gave_up) *reinterpret_cast<volatile uint32_t *>(a.gave_up) = 1u;
+                }
             }
         }
         __syncthreads();                 // every warp is done with the query's shared memory
+        if (*gave_up) {                  // the same for all: nobody waits on a barrier now
+            __syncthreads();
+            if (threadIdx.x == 0) {
+                for (uint32_t i = 0; i < 2u * nexp; ++i) {
+                    team_bar_inval(bar0 + 8u * i);
+                    team_bar_init(bar0 + 8u * i);
+                }
+                asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
+                *gave_up = 0u;
+            }
+            phase = 0;
+            __syncthreads();
+        }
     }
 }
 
@@ -872,7 +901,12 @@ template <int MODE> cudaError_t launch_team(const SearchArgs &a, int dtype, size
     cudaError_t e;
     if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
     if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
-    const uint32_t nexp = a.phase_cycles || a.ncodes ? 0u : team_expanders(a, MODE, sms);
+    const bool one = a.phase_cycles || a.ncodes;
+    const uint32_t nexp = a.form ? a.form - 1u : one ? 0u : team_expanders(a, MODE, sms);
+    if (a.form > 1u && (one || nexp > kTeamMaxExpanders ||
+                        TeamLayout(a.M, a.log2z, a.L, a.k, a.d, a.R, MODE, nexp).total > 227u * 1024u))
+        return cudaErrorInvalidValue;            // asked for by name, but not possible here
+    if (a.form_out) *a.form_out = 1u + nexp;
     if (nexp == 0) return launch_mode<MODE>(a, dtype, smem, st);
     const bool narrow = a.d <= 128, wide_r = a.R > 64;
 #define BANG_DISPATCH(DT)                                                                                    \

@@ -50,6 +50,7 @@ struct Request {
     Clock::time_point t_submit, t_done;
     bool done = false;
     int status = BANG_OK;
+    bool gave_up = false;                  // status BANG_ECUDA: a wait inside the search did
 };
 
 // A launch in flight: its arena region and the requests it carries.
@@ -60,10 +61,13 @@ struct Launch {
     bool finished = false;
 };
 
+constexpr size_t kWord = 64;               // page-locked bytes per stream for its launches' give-up flag
+
 struct Stream {
     cudaStream_t stream = nullptr;
     cudaEvent_t done = nullptr;
     std::shared_ptr<Launch> launch;        // null: free
+    volatile uint32_t *gave_up = nullptr;  // page-locked: a wait inside the launch's search gave up
     bang_server *srv = nullptr;            // for the completion host function
 };
 
@@ -76,7 +80,8 @@ struct bang_server {
     size_t esz = 1;
     int device = 0;
     size_t cap = 0;                        // arena bytes
-    unsigned char *d_arena = nullptr, *h_arena = nullptr;
+    unsigned char *d_arena = nullptr, *h_arena = nullptr, *h_words = nullptr;
+    bang::SearchForm form;                 // of every launch
     std::deque<std::shared_ptr<Launch>> regions;   // live regions in allocation order
     std::vector<Stream> streams;
     std::mutex mu;
@@ -180,8 +185,11 @@ int start_launch(bang_server *s, Stream &st, Launch &ln)
     p.mode = s->cfg.mode;
     p.bloom_log2 = s->cfg.bloom_log2;
     p.early_codes = s->cfg.early_codes;
+    bang::SearchForm form = s->form;
+    form.gave_up = const_cast<uint32_t *>(st.gave_up);
+    *st.gave_up = 0u;
     int rc = bang::search_batched(s->ix, dv.q, nq, dv.k, dv.L, s->cfg.k_max, s->cfg.L_max, &p, dv.ids,
-                                  dv.dist, st.stream, true);
+                                  dv.dist, st.stream, form);
     if (rc != BANG_OK) return rc;
     const size_t out_bytes = 2 * up(static_cast<size_t>(nq) * s->cfg.k_max * 4);   // ids, distances
     cudaMemcpyAsync(h.ids, dv.ids, out_bytes, cudaMemcpyDeviceToHost, st.stream);
@@ -204,7 +212,8 @@ void finish_launch(bang_server *s, Stream &st, int status)
         r->dist.assign(h.dist + static_cast<size_t>(off) * km, h.dist + static_cast<size_t>(off + r->nq) * km);
         off += r->nq;
         r->t_done = now;
-        r->status = status;
+        r->status = status != BANG_OK ? status : *st.gave_up ? BANG_ECUDA : BANG_OK;
+        r->gave_up = status == BANG_OK && *st.gave_up;
         r->done = true;
     }
     ln.batch.clear();
@@ -270,7 +279,8 @@ void release_all(bang_server *s)
     s->streams.clear();
     if (s->d_arena) cudaFree(s->d_arena);
     if (s->h_arena) cudaFreeHost(s->h_arena);
-    s->d_arena = s->h_arena = nullptr;
+    if (s->h_words) cudaFreeHost(s->h_words);
+    s->d_arena = s->h_arena = s->h_words = nullptr;
 }
 
 }  // namespace
@@ -301,7 +311,9 @@ int bang_server_start(bang_index *ix, const bang_server_config *cfg, bang_server
                             : cfg->streams * batch_bytes(s.get(), cfg->max_batch);
     if (s->cap < batch_bytes(s.get(), 1))
         return sfail(BANG_EINVAL, "bang_server_start: mem_bytes holds not even one query");
-    if (cudaMalloc(&s->d_arena, s->cap) != cudaSuccess || cudaHostAlloc(&s->h_arena, s->cap, 0) != cudaSuccess) {
+    s->form.overlapped = true;
+    if (cudaMalloc(&s->d_arena, s->cap) != cudaSuccess || cudaHostAlloc(&s->h_arena, s->cap, 0) != cudaSuccess ||
+        cudaHostAlloc(&s->h_words, cfg->streams * kWord, 0) != cudaSuccess) {
         cudaGetLastError();
         release_all(s.get());
         return sfail(BANG_ENOMEM, "bang_server_start: the arena does not fit; lower mem_bytes");
@@ -309,6 +321,7 @@ int bang_server_start(bang_index *ix, const bang_server_config *cfg, bang_server
     s->streams.resize(cfg->streams);
     for (Stream &st : s->streams) {
         st.srv = s.get();
+        st.gave_up = reinterpret_cast<uint32_t *>(s->h_words + kWord * static_cast<size_t>(&st - s->streams.data()));
         if (cudaStreamCreateWithFlags(&st.stream, cudaStreamNonBlocking) != cudaSuccess ||
             cudaEventCreateWithFlags(&st.done, cudaEventDisableTiming) != cudaSuccess) {
             cudaGetLastError();
@@ -383,11 +396,23 @@ int bang_server_wait(bang_server *s, uint64_t ticket, int32_t timeout_ms, uint32
         return sfail(BANG_ETIMEOUT, "bang_server_wait: request not finished in time");
     s->live.erase(it);
     lk.unlock();
-    if (r->status != BANG_OK) return sfail(r->status, "bang_server_wait: the batch failed");
+    if (r->status != BANG_OK)
+        return sfail(r->status, r->gave_up ? "bang_server_wait: a bounded wait inside the batch's search gave up"
+                                           : "bang_server_wait: the batch failed");
     if (out_ids) std::memcpy(out_ids, r->ids.data(), r->ids.size() * 4);
     if (out_dist) std::memcpy(out_dist, r->dist.data(), r->dist.size() * 4);
     if (latency_ms)
         *latency_ms = std::chrono::duration<double, std::milli>(r->t_done - r->t_submit).count();
+    return BANG_OK;
+}
+
+int bang_internal_server_form(bang_server *s, uint32_t form, long long wait_cycles, uint32_t mute)
+{
+    if (!s) return sfail(BANG_EINVAL, "bang_internal_server_form: NULL server");
+    std::lock_guard<std::mutex> lk(s->mu);
+    s->form.form = form;
+    s->form.wait_cycles = wait_cycles;
+    s->form.mute = mute;
     return BANG_OK;
 }
 
