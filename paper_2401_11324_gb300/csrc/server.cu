@@ -259,7 +259,10 @@ void dispatch_loop(bang_server *s)
             lk.unlock();
             int rc = start_launch(s, st, *ln);
             lk.lock();
-            if (rc != BANG_OK) finish_launch(s, st, rc);
+            if (rc != BANG_OK) {
+                finish_launch(s, st, rc);
+                s->cv_done.notify_all();
+            }
             progressed = true;
         }
         bool any_busy = false;

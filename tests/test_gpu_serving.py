@@ -2,11 +2,12 @@
 while others run are packed into overlapping launches, and every request's
 result equals the same request searched alone (FP32 form: bit for bit)."""
 import threading
+import time
 
 import numpy as np
 import pytest
 
-from tests import cases
+from tests import cases, forms
 
 torch = pytest.importorskip("torch")
 pytestmark = pytest.mark.gpu
@@ -161,6 +162,25 @@ def test_server_where_only_the_one_warp_form_fits(Lmax):
         for i, t in zip((0, 20, 40), tickets):
             ids, dist, _ = srv.wait(t, 20_000)
             assert (ids == want[0][i:i + 20]).all() and (dist == want[1][i:i + 20]).all()
+    finally:
+        srv.stop()
+        ix.close()
+
+
+def test_a_launch_that_is_refused_wakes_its_waiters():
+    # three expanders do not fit beside this layout (test above): every launch
+    # is refused, and the requests end at once, whether they are waited for
+    # before or after
+    w = cases.clustered(n=5_000, nq=60, ncomp=4, dtype="f32", d=96, M=96, R=32, centre="uniform255")
+    ix = bang.Index(w["base"], w["codebook"], w["codes"], w["adj"], w["medoid"], 96)
+    srv = bang.Server(ix, 10, 96, max_batch=32, streams=2, bloom_log2=20)
+    try:
+        forms.server_form(srv, 4)
+        for _ in range(20):
+            began = time.perf_counter()
+            with pytest.raises(bang.BangError) as e:
+                srv.wait(srv.submit(w["queries"][:20], np.full(20, 10, np.uint32), np.full(20, 32, np.uint32)), 20_000)
+            assert e.value.code == bang.BANG_ECUDA and time.perf_counter() - began < 10
     finally:
         srv.stop()
         ix.close()
