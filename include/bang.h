@@ -427,8 +427,10 @@ int bang_build_pq(int device, const void *base, bang_dtype dtype, uint64_t n, ui
  * sum rounded; sorted by (distance, id), padded with 0xFFFFFFFF / +inf when
  * n < k.  base (n*d) and queries (nq*d) host or device, of dtype; out_ids and
  * out_dist (nq*k) both host or both device.  k <= 256, d <= 4096.  Allocates
- * device scratch (about nq*(k*400 + 3000) bytes, up to 0.9 GB of converted rows, and copies of host
- * inputs) and blocks until done. */
+ * copies of host inputs and scratch on the device: about k*400 + 3000 bytes for
+ * each of up to 65,536 queries at a time, and up to 0.9 GB of converted rows;
+ * where that does not fit, fewer queries at a time and no converted rows, which
+ * is slower.  Blocks until done. */
 int bang_ground_truth(int device, const void *base, const void *queries, bang_dtype dtype, uint64_t n,
                       uint32_t nq, uint32_t d, uint32_t k, uint32_t *out_ids, double *out_dist,
                       void *stream);

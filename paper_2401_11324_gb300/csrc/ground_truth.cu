@@ -44,6 +44,7 @@ constexpr uint32_t kMaxK = 256;
 constexpr uint32_t kTileQ = 128;         // at most this many queries per CTA in pass 2
 constexpr uint32_t kSample = 1024;       // points of the first threshold
 constexpr uint64_t kQueries = 1u << 16;  // queries at a time
+constexpr uint32_t kLeastQueries = 64;   // at least, where memory is short
 constexpr uint32_t kLevel = 16;          // each further level streams over this many times as many
 
 struct GtArgs {
@@ -402,13 +403,20 @@ struct TcLevel {
         }
         const uint32_t qt = (nq + gt_tc::kTileP - 1u) / gt_tc::kTileP;
         const uint64_t pt = ((n < gt_tc::kTcPoints ? n : gt_tc::kTcPoints) + gt_tc::kTileP - 1u) / gt_tc::kTileP;
-        cudaError_t e;
-        if ((e = qtiles.alloc(static_cast<uint64_t>(qt) * nblk * gt_tc::kBlock)) != cudaSuccess) return e;
-        if ((e = ptiles.alloc(pt * nblk * gt_tc::kBlock)) != cudaSuccess) return e;
-        if ((e = pnorm.alloc(pt * gt_tc::kTileP)) != cudaSuccess) return e;
-        if ((e = lim.alloc(nq)) != cudaSuccess) return e;
-        if ((e = qq.alloc(nq)) != cudaSuccess) return e;
-        if ((e = flags.alloc(2)) != cudaSuccess) return e;
+        cudaError_t e = qtiles.alloc(static_cast<uint64_t>(qt) * nblk * gt_tc::kBlock);
+        if (e == cudaSuccess) e = ptiles.alloc(pt * nblk * gt_tc::kBlock);
+        if (e == cudaSuccess) e = pnorm.alloc(pt * gt_tc::kTileP);
+        if (e == cudaSuccess) e = lim.alloc(nq);
+        if (e == cudaSuccess) e = qq.alloc(nq);
+        if (e == cudaSuccess) e = flags.alloc(2);
+        if (e == cudaErrorMemoryAllocation) {      // up to 0.9 GB that the other form does without
+            cudaGetLastError();
+            qtiles.alloc(0);
+            ptiles.alloc(0);
+            on = false;
+            return cudaSuccess;
+        }
+        if (e != cudaSuccess) return e;
         if ((e = cudaMemsetAsync(flags.p, 0, 8, st)) != cudaSuccess) return e;
         // the limit belongs to the kernel and outlasts this call: the same for every
         // thread, as others launch with theirs between this call's levels
@@ -482,6 +490,107 @@ int gtfail(int code, const std::string &m)
         }                                                                                   \
     } while (0)
 
+namespace {
+
+// The k nearest of n points (B) for m queries (Q), all on the device but the
+// results where they go to the host.
+int truth_of(int device, const void *B, const void *Q, bang_dtype dtype, uint64_t n, uint32_t m, uint32_t d, uint32_t k,
+             uint32_t tileq, bool tensor, uint32_t *ids, double *dist, bool dev_out, cudaStream_t st)
+{
+    const size_t esz = dtype == BANG_F32 ? 4 : 1;
+    DArr<double> thr, cd, odist;
+    DArr<uint32_t> cnt, ci, oids;
+    GT_TRY(thr.alloc(m));
+    GT_TRY(cnt.alloc(m));
+    GtArgs g;
+    std::memset(&g, 0, sizeof g);
+    g.base = B;
+    g.queries = Q;
+    g.dtype = dtype;
+    g.nq = m;
+    g.d = d;
+    g.k = k;
+    g.thr_out = thr.p;
+    g.thr = thr.p;
+    g.cnt = cnt.p;
+    g.tileq = tileq;
+    {
+        const uintptr_t ab = reinterpret_cast<uintptr_t>(B), aq = reinterpret_cast<uintptr_t>(Q);
+        g.words = dtype != BANG_F32 && d % 4 == 0 && ab % 4 == 0 && aq % 4 == 0;
+        g.regrow = dtype != BANG_F32 && d % 16 == 0 && d <= 128 && ab % 16 == 0;
+    }
+    g.n = n < kSample ? n : kSample;
+    g.stride = n / g.n;
+    sample_threshold<<<(m + kSampleWarps - 1) / kSampleWarps, kSampleWarps * kW, 0, st>>>(g);
+    GT_TRY(cudaGetLastError());
+    int sms = 0;
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, device);
+    const uint32_t tiles = (m + tileq - 1) / tileq;
+    std::vector<uint32_t> c(m);
+    uint64_t cap = 0;
+    TcLevel tc(B, Q, dtype, d, m, sms);
+    tc.on = tc.on && tensor;
+    GT_TRY(tc.prepare(n, st));
+    for (uint64_t seen = g.n;; seen = g.n) {
+        g.n = seen < n / kLevel ? seen * kLevel : n;     // the last level takes every point
+        g.stride = n / g.n;
+        // expected list length about k * (points now / points before); room for twice that, then the longest
+        uint64_t room = 2ull * k * ((g.n + seen - 1) / seen) + 256;
+        for (int attempt = 0;; ++attempt) {
+            if (room > cap) {
+                GT_TRY(cd.alloc(room * m));
+                GT_TRY(ci.alloc(room * m));
+                cap = room;
+            }
+            GT_TRY(cudaMemsetAsync(cnt.p, 0, m * 4, st));
+            g.cd = cd.p;
+            g.ci = ci.p;
+            g.cap = cap;
+            if (tc.on && g.n >= kTcLeast) GT_TRY(tc.collect(g, st));
+            else {
+                // fewer queries a block where the level's points alone would not fill the GPU
+                const uint64_t have = (g.n + 255u) / 256u * tiles, want = 4ull * sms;
+                g.tileq = have < want ? static_cast<uint32_t>(std::max<uint64_t>(1u, tileq * have / want)) : tileq;
+                const uint32_t ty = (m + g.tileq - 1u) / g.tileq;
+                const uint32_t tx = static_cast<uint32_t>((static_cast<uint64_t>(sms) * 8 + ty - 1) / ty) + 1;
+                collect<<<dim3(tx, ty), 256, g.tileq * d * esz, st>>>(g);
+            }
+            GT_TRY(cudaGetLastError());
+            GT_TRY(cudaMemcpyAsync(c.data(), cnt.p, m * 4, cudaMemcpyDeviceToHost, st));
+            if (tc.on) GT_TRY(cudaMemcpyAsync(tc.state, tc.flags.p, sizeof tc.state, cudaMemcpyDeviceToHost, st));
+            GT_TRY(cudaStreamSynchronize(st));
+            if (tc.on && tc.state[1]) return gtfail(BANG_ETIMEOUT, "bang_ground_truth: a tensor-core wait gave up");
+            if (tc.on && tc.state[0]) {          // values the filter cannot bound: this level again without it
+                tc.on = false;
+                --attempt;
+                continue;
+            }
+            room = *std::max_element(c.begin(), c.end());
+            if (room <= cap) break;
+            if (attempt == 1) return gtfail(BANG_ECUDA, "bang_ground_truth: candidate lists kept growing");
+        }
+        if (g.n == n) break;
+        kth_threshold<<<(m + kKthWarps - 1) / kKthWarps, kKthWarps * kW, 0, st>>>(g);
+        GT_TRY(cudaGetLastError());
+    }
+    if (!dev_out) {
+        GT_TRY(oids.alloc(static_cast<uint64_t>(m) * k));
+        GT_TRY(odist.alloc(static_cast<uint64_t>(m) * k));
+    }
+    g.out_ids = dev_out ? ids : oids.p;
+    g.out_dist = dev_out ? dist : odist.p;
+    select_k<<<(m + kKthWarps - 1) / kKthWarps, kKthWarps * kW, 0, st>>>(g);
+    GT_TRY(cudaGetLastError());
+    if (!dev_out) {
+        GT_TRY(cudaMemcpyAsync(ids, oids.p, static_cast<uint64_t>(m) * k * 4, cudaMemcpyDeviceToHost, st));
+        GT_TRY(cudaMemcpyAsync(dist, odist.p, static_cast<uint64_t>(m) * k * 8, cudaMemcpyDeviceToHost, st));
+    }
+    GT_TRY(cudaStreamSynchronize(st));
+    return BANG_OK;
+}
+
+}  // namespace
+
 extern "C" int bang_ground_truth(int device, const void *base, const void *queries, bang_dtype dtype,
                                  uint64_t n, uint32_t nq, uint32_t d, uint32_t k, uint32_t *out_ids,
                                  double *out_dist, void *stream)
@@ -521,99 +630,25 @@ extern "C" int bang_ground_truth(int device, const void *base, const void *queri
         Q = dq.p;
     }
     const bool dev_out = is_dev(out_ids);
-    // kQueries queries at a time: the candidate lists are sized for one block
-    for (uint64_t q0 = 0; q0 < nq; q0 += kQueries) {
-        const uint32_t m = static_cast<uint32_t>(nq - q0 < kQueries ? nq - q0 : kQueries);
-        const void *Qb = static_cast<const unsigned char *>(Q) + q0 * d * esz;
-        uint32_t *ids = out_ids + q0 * k;
-        double *dist = out_dist + q0 * k;
-        DArr<double> thr, cd, odist;
-        DArr<uint32_t> cnt, ci, oids;
-        GT_TRY(thr.alloc(m));
-        GT_TRY(cnt.alloc(m));
-        GtArgs g;
-        std::memset(&g, 0, sizeof g);
-        g.base = B;
-        g.queries = Qb;
-        g.dtype = dtype;
-        g.nq = m;
-        g.d = d;
-        g.k = k;
-        g.thr_out = thr.p;
-        g.thr = thr.p;
-        g.cnt = cnt.p;
-        g.tileq = tileq;
-        {
-            const uintptr_t ab = reinterpret_cast<uintptr_t>(B), aq = reinterpret_cast<uintptr_t>(Qb);
-            g.words = dtype != BANG_F32 && d % 4 == 0 && ab % 4 == 0 && aq % 4 == 0;
-            g.regrow = dtype != BANG_F32 && d % 16 == 0 && d <= 128 && ab % 16 == 0;
+    // kQueries queries at a time, fewer where their candidate lists do not fit
+    // (they are longer than those of a single pass over the points), in the end
+    // without the tensor cores' operands
+    uint64_t block = kQueries;
+    bool tensor = true;
+    for (uint64_t q0 = 0; q0 < nq;) {
+        const uint32_t m = static_cast<uint32_t>(nq - q0 < block ? nq - q0 : block);
+        const int rc = truth_of(device, B, static_cast<const unsigned char *>(Q) + q0 * d * esz, dtype, n, m, d, k, tileq,
+                                tensor, out_ids + q0 * k, out_dist + q0 * k, dev_out, st);
+        if (rc == BANG_ENOMEM && m > kLeastQueries) {
+            block = (m + 1u) / 2u;
+            continue;
         }
-        g.n = n < kSample ? n : kSample;
-        g.stride = n / g.n;
-        sample_threshold<<<(m + kSampleWarps - 1) / kSampleWarps, kSampleWarps * kW, 0, st>>>(g);
-        GT_TRY(cudaGetLastError());
-        int sms = 0;
-        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, device);
-        const uint32_t tiles = (m + tileq - 1) / tileq;
-        std::vector<uint32_t> c(m);
-        uint64_t cap = 0;
-        TcLevel tc(B, Qb, dtype, d, m, sms);
-        GT_TRY(tc.prepare(n, st));
-        for (uint64_t seen = g.n;; seen = g.n) {
-            g.n = seen < n / kLevel ? seen * kLevel : n;     // the last level takes every point
-            g.stride = n / g.n;
-            // expected list length about k * (points now / points before); room for twice that, then the longest
-            uint64_t room = 2ull * k * ((g.n + seen - 1) / seen) + 256;
-            for (int attempt = 0;; ++attempt) {
-                if (room > cap) {
-                    GT_TRY(cd.alloc(room * m));
-                    GT_TRY(ci.alloc(room * m));
-                    cap = room;
-                }
-                GT_TRY(cudaMemsetAsync(cnt.p, 0, m * 4, st));
-                g.cd = cd.p;
-                g.ci = ci.p;
-                g.cap = cap;
-                if (tc.on && g.n >= kTcLeast) GT_TRY(tc.collect(g, st));
-                else {
-                    // fewer queries a block where the level's points alone would not fill the GPU
-                    const uint64_t have = (g.n + 255u) / 256u * tiles, want = 4ull * sms;
-                    g.tileq = have < want ? static_cast<uint32_t>(std::max<uint64_t>(1u, tileq * have / want)) : tileq;
-                    const uint32_t ty = (m + g.tileq - 1u) / g.tileq;
-                    const uint32_t tx = static_cast<uint32_t>((static_cast<uint64_t>(sms) * 8 + ty - 1) / ty) + 1;
-                    collect<<<dim3(tx, ty), 256, g.tileq * d * esz, st>>>(g);
-                }
-                GT_TRY(cudaGetLastError());
-                GT_TRY(cudaMemcpyAsync(c.data(), cnt.p, m * 4, cudaMemcpyDeviceToHost, st));
-                if (tc.on) GT_TRY(cudaMemcpyAsync(tc.state, tc.flags.p, sizeof tc.state, cudaMemcpyDeviceToHost, st));
-                GT_TRY(cudaStreamSynchronize(st));
-                if (tc.on && tc.state[1]) return gtfail(BANG_ETIMEOUT, "bang_ground_truth: a tensor-core wait gave up");
-                if (tc.on && tc.state[0]) {          // values the filter cannot bound: this level again without it
-                    tc.on = false;
-                    --attempt;
-                    continue;
-                }
-                room = *std::max_element(c.begin(), c.end());
-                if (room <= cap) break;
-                if (attempt == 1) return gtfail(BANG_ECUDA, "bang_ground_truth: candidate lists kept growing");
-            }
-            if (g.n == n) break;
-            kth_threshold<<<(m + kKthWarps - 1) / kKthWarps, kKthWarps * kW, 0, st>>>(g);
-            GT_TRY(cudaGetLastError());
+        if (rc == BANG_ENOMEM && tensor) {
+            tensor = false;
+            continue;
         }
-        if (!dev_out) {
-            GT_TRY(oids.alloc(static_cast<uint64_t>(m) * k));
-            GT_TRY(odist.alloc(static_cast<uint64_t>(m) * k));
-        }
-        g.out_ids = dev_out ? ids : oids.p;
-        g.out_dist = dev_out ? dist : odist.p;
-        select_k<<<(m + kKthWarps - 1) / kKthWarps, kKthWarps * kW, 0, st>>>(g);
-        GT_TRY(cudaGetLastError());
-        if (!dev_out) {
-            GT_TRY(cudaMemcpyAsync(ids, oids.p, static_cast<uint64_t>(m) * k * 4, cudaMemcpyDeviceToHost, st));
-            GT_TRY(cudaMemcpyAsync(dist, odist.p, static_cast<uint64_t>(m) * k * 8, cudaMemcpyDeviceToHost, st));
-        }
-        GT_TRY(cudaStreamSynchronize(st));
+        if (rc != BANG_OK) return rc;
+        q0 += m;
     }
     return BANG_OK;
 }

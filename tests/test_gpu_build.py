@@ -223,3 +223,25 @@ def test_pq_build_where_fp32_is_not_enough(dt, d, M, ns, what):
     cb, codes = bang.bang_build_pq(X, M, sample, init, 3)
     assert (cb.view(np.uint32) == cb_ref.view(np.uint32)).all()
     assert (codes == codes_ref).all()
+
+
+@pytest.mark.parametrize("dt,left", [("u8", 3 << 29), ("f32", 3 << 28)])
+def test_ground_truth_where_memory_is_short(dt, left):
+    # the candidate lists of 60,000 queries at k = 256 want 6 GB, the rows'
+    # operands for the tensor cores up to 0.9 GB more; the lists of a single
+    # pass were 0.6 GB.  With 1.5 and 0.75 GB left the same result comes, fewer
+    # queries at a time
+    nq, n, d, k = 60_000, 20_000, 16, 256
+    g = torch.Generator(device="cuda").manual_seed(1)
+    X = torch.randint(0, 256, (n, d), generator=g, device="cuda")
+    X = X.to(torch.uint8 if dt == "u8" else torch.float32)
+    Q = torch.randint(0, 256, (nq, d), generator=g, device="cuda").to(X.dtype)
+    want = bang.bang_ground_truth(X, Q, k)
+    torch.cuda.empty_cache()
+    hog = torch.empty(torch.cuda.mem_get_info()[0] - left, dtype=torch.uint8, device="cuda")
+    try:
+        got = bang.bang_ground_truth(X, Q, k)
+    finally:
+        del hog
+        torch.cuda.empty_cache()
+    assert (got[0] == want[0]).all() and (got[1] == want[1]).all()
