@@ -116,7 +116,7 @@ struct SearchArgs {
     // Team form: what becomes of its bounded waits (search_team.cuh).
     long long wait_cycles;    // SM cycles until one gives up (0: kTeamWaitCycles)
     uint32_t *gave_up;        // device-accessible or null: set to 1 when one did
-    uint32_t mute;            // 1 + the query whose first expander answers nothing (0: none), for tests
+    uint32_t mute;            // 1 + the query whose first request gets lost (0: none), for tests
     uint32_t ntab;            // kModeF32Lazy: subspaces (the first ones) whose entries stay in a table
 };
 

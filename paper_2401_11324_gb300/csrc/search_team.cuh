@@ -92,6 +92,21 @@ __device__ __forceinline__ void team_bar_inval(uint32_t bar)
 {
     asm volatile("mbarrier.inval.shared::cta.b64 [%0];\n" ::"r"(bar) : "memory");
 }
+// New barriers, by all threads together.  Out of line, so that the search's
+// loops are compiled as if it were not there.
+static __device__ __noinline__ void team_start_over(uint32_t bar0, uint32_t count, volatile uint32_t *gave_up)
+{
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        for (uint32_t i = 0; i < count; ++i) {
+            team_bar_inval(bar0 + 8u * i);
+            team_bar_init(bar0 + 8u * i);
+        }
+        asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
+        *gave_up = 0u;
+    }
+    __syncthreads();
+}
 __device__ __forceinline__ void team_arrive(uint32_t bar)
 {
     asm volatile("{\n\t.reg .b64 t;\n\tmbarrier.arrive.release.cta.shared::cta.b64 t, [%0];\n\t}\n" ::"r"(bar)
@@ -109,12 +124,12 @@ __device__ __forceinline__ bool team_test(uint32_t bar, uint32_t parity)
         : "memory");
     return ok != 0u;
 }
-// Whole warp; false when the wait gave up, after about `limit` cycles.
-__device__ __forceinline__ bool team_wait(uint32_t bar, uint32_t parity, long long limit)
+// One lane's wait; false when it gave up, after about `limit` cycles.
+__device__ __forceinline__ bool team_wait_lane(uint32_t bar, uint32_t parity, long long limit)
 {
     uint32_t ok = 0;
     long long began = 0;
-    for (uint32_t i = 0; !ok; ++i) {
+    for (uint32_t i = 0;; ++i) {
         asm volatile(
             "{\n\t.reg .pred P;\n\t"
             "mbarrier.try_wait.parity.acquire.cta.shared::cta.b64 P, [%1], %2;\n\t"
@@ -122,11 +137,25 @@ __device__ __forceinline__ bool team_wait(uint32_t bar, uint32_t parity, long lo
             : "=r"(ok)
             : "r"(bar), "r"(parity)
             : "memory");
-        if (ok) break;
+        if (ok) return true;
         if (i == 0) began = clock64();
-        else if (clock64() - began > limit) break;
+        else if (clock64() - began > limit) return false;
     }
-    return __all_sync(0xFFFFFFFFu, ok != 0u) != 0;
+}
+// Whole warp: one answer for all lanes.
+__device__ __forceinline__ bool team_wait(uint32_t bar, uint32_t parity, long long limit)
+{
+    return __all_sync(0xFFFFFFFFu, team_wait_lane(bar, parity, limit)) != 0;
+}
+// The same, and with `ask` whether another barrier's phase is over by then (bit
+// 1 beside bit 0): each lane asks for itself while the other side may arrive at
+// any moment, so that answer needs the vote as well.  One vote for both.
+__device__ __forceinline__ uint32_t team_wait_ask(uint32_t bar, uint32_t parity, long long limit, bool ask,
+                                                  uint32_t bar2, uint32_t parity2)
+{
+    uint32_t got = team_wait_lane(bar, parity, limit) ? 1u : 0u;
+    if (ask && team_test(bar2, parity2)) got |= 2u;
+    return __reduce_and_sync(0xFFFFFFFFu, got);
 }
 
 __device__ __forceinline__ bool team_seen(const volatile uint32_t *bloom, uint32_t p1, uint32_t p2)
@@ -289,7 +318,6 @@ __global__ void __maxnreg__(team_regs(DCH, MODE)) team_kernel(const SearchArgs a
     uint32_t *qw = reinterpret_cast<uint32_t *>(smem + lay.off_qw);
     volatile uint32_t *head = reinterpret_cast<volatile uint32_t *>(smem + lay.off_head);   // 3 words per slot
     volatile uint32_t *ticket = head + 3u * nexp, *gave_up = ticket + 1;
-    const long long limit = a.wait_cycles ? a.wait_cycles : kTeamWaitCycles;
     const uint32_t bar0 = team_smem_addr(smem + lay.off_bar);   // slot e: request at +16e, result at +16e+8
     float *qv = reinterpret_cast<float *>(smem + lay.off_q);
     uint32_t *offs = reinterpret_cast<uint32_t *>(smem + lay.off_offs);
@@ -373,7 +401,7 @@ __global__ void __maxnreg__(team_regs(DCH, MODE)) team_kernel(const SearchArgs a
             uint32_t *db = ids + rw;
             const uint32_t req = bar0 + 16u * e;
             for (;;) {
-                if (!team_wait(req, phase, limit) || (e == 0u && q + 1u == a.mute)) {
+                if (!team_wait(req, phase, a.wait_cycles)) {
                     if (lane == 0) *gave_up = 1u;
                     break;
                 }
@@ -486,7 +514,8 @@ __global__ void __maxnreg__(team_regs(DCH, MODE)) team_kernel(const SearchArgs a
                     __syncwarp();
                 }
             };
-            if (have_next) post(0u, ukey);
+            if (have_next && q + 1u != a.mute) post(0u, ukey);
+            else if (lane == 0) sid = have_next ? key_id(ukey) : kNone;      // (tests: a request that gets lost)
 
             while (have_next) {
                 if (iters >= iter_cap) {
@@ -497,19 +526,18 @@ __global__ void __maxnreg__(team_regs(DCH, MODE)) team_kernel(const SearchArgs a
                 // (one bit at most: the leading-zero count is half of __ffs)
                 const uint32_t se = 31u - __clz(__ballot_sync(0xFFFFFFFFu, sid == u));
                 const uint32_t s2 = 31u - __clz(__ballot_sync(0xFFFFFFFFu, sid == u2));     // ~0: in no slot
-                if (!team_wait(result(se), (phase >> se) & 1u, limit)) {
-                    status = 3;
-                    break;
-                }
                 // Two expansions at once: the entry after u* is next after it
                 // unless one of u*'s new neighbours is nearer.  When its slot
                 // is ready too and both nodes' neighbours fit the warp, they
                 // are filtered together, u*'s first.
-                // (Each lane asks for itself while the expander may arrive at
-                // any moment: the vote makes one answer of it, which the
-                // branches and votes below need.)
                 bool pair = lkey != ~0ull && s2 < nexp && both3 && iters + 1u < iter_cap;
-                if (pair) pair = __all_sync(0xFFFFFFFFu, team_test(result(s2), (phase >> s2) & 1u)) != 0;
+                const uint32_t got = team_wait_ask(result(se), (phase >> se) & 1u, a.wait_cycles, pair, result(s2),
+                                                   (phase >> (s2 & 31u)) & 1u);
+                if (!(got & 1u)) {
+                    status = 3;
+                    break;
+                }
+                pair = (got & 2u) != 0u;
                 const uint32_t m = head[3u * se + 1u], xd = head[3u * se + 2u];
                 uint32_t m2 = 0, xd2 = 0;
                 if (pair) {
@@ -769,7 +797,7 @@ __global__ void __maxnreg__(team_regs(DCH, MODE)) team_kernel(const SearchArgs a
             // ---- end of the query: the expanders finish and stop
             for (uint32_t e = 0; e < nexp; ++e) {
                 if (__shfl_sync(0xFFFFFFFFu, sid, static_cast<int>(e)) != kNone) {
-                    if (!team_wait(result(e), (phase >> e) & 1u, limit)) status = 3;
+                    if (!team_wait(result(e), (phase >> e) & 1u, a.wait_cycles)) status = 3;
                     phase ^= 1u << e;
                 }
                 if (static_cast<uint32_t>(lane) == e) {
@@ -814,17 +842,8 @@ __global__ void __maxnreg__(team_regs(DCH, MODE)) team_kernel(const SearchArgs a
         }
         __syncthreads();                 // every warp is done with the query's shared memory
         if (*gave_up) {                  // the same for all: nobody waits on a barrier now
-            __syncthreads();
-            if (threadIdx.x == 0) {
-                for (uint32_t i = 0; i < 2u * nexp; ++i) {
-                    team_bar_inval(bar0 + 8u * i);
-                    team_bar_init(bar0 + 8u * i);
-                }
-                asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
-                *gave_up = 0u;
-            }
+            team_start_over(bar0, 2u * nexp, gave_up);
             phase = 0;
-            __syncthreads();
         }
     }
 }
@@ -895,8 +914,10 @@ cudaError_t launch_team_one(const SearchArgs &a, uint32_t nexp, int sms, cudaStr
 // Launch of one mode.  The one-warp form (search_kernel.cuh) stays where it is
 // faster (above) and for what the team form does not do: the per-phase clock
 // and the neighbour-code layout.
-template <int MODE> cudaError_t launch_team(const SearchArgs &a, int dtype, size_t smem, cudaStream_t st)
+template <int MODE> cudaError_t launch_team(const SearchArgs &args, int dtype, size_t smem, cudaStream_t st)
 {
+    SearchArgs a = args;
+    if (a.wait_cycles == 0) a.wait_cycles = kTeamWaitCycles;
     int dev = 0, sms = 0;
     cudaError_t e;
     if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
