@@ -654,8 +654,20 @@ template <bool ON> struct PhaseClock {
 // (every neighbour's row arrives with the node); 2 = every neighbour's row
 // requested from the codes as soon as the node's row arrives, so that the
 // filter runs while they are in flight (rows of at most 32 bytes).
+// Queries an SM's registers have to hold (16,384 in each quarter of it); 0: as
+// they come.  Exact distances of integer rows, a lane per row: left alone, the
+// compiler takes 84 registers a thread (112 with four neighbours a lane), which
+// hold 20 (16) queries; 72 (80) hold 28 (24) and spill a word at most.  10,000 u8
+// queries at L = 48, 200,000 points, HBM: 618 -> 579 us; 6,000 int8 queries,
+// rows of 68 neighbours, L = 64: 669 -> 500; 1,233 u8 queries at L = 366 from
+// host memory: 3,920 -> 3,000.
+constexpr int least_queries(int dt, int rpl, int dch, int mode, bool ph)
+{
+    return mode == kModeExact && dt != 2 && dch == 1 && !ph ? (rpl == 2 ? 28 : 24) : 0;
+}
+
 template <int DT, int RPL, int DCH, int MODE, int CS, bool PH>
-__global__ void __launch_bounds__(32) search_kernel(const SearchArgs a)
+__global__ void __launch_bounds__(32, least_queries(DT, RPL, DCH, MODE, PH)) search_kernel(const SearchArgs a)
 {
     using E = typename Elem<DT>::T;
     constexpr bool kPQ = MODE != kModeExact;

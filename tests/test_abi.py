@@ -113,3 +113,15 @@ def test_host_alloc_aligned_zeroed_and_freed(lib):
     assert lib.bang_host_alloc(0, ctypes.byref(p)) == bang.BANG_EINVAL
     a = bang.host_empty((300, 7), np.float32)
     assert a.shape == (300, 7) and a.dtype == np.float32 and not a.any()
+
+
+def test_exact_search_fits_its_registers(lib):
+    # one warp per query, integer rows, two and four neighbours a lane: 72 and
+    # 80 registers a thread hold 28 and 24 queries an SM
+    out = subprocess.check_output(["cuobjdump", "-res-usage", bbuild.LIB], text=True)
+    for dt in (0, 1):
+        for rpl, most in ((2, 72), (4, 80)):
+            name = "search_kernelILi%dELi%dELi1ELi2ELi0ELb0E" % (dt, rpl)
+            use = re.search(r"Function \S*%s\S*:\s*REG:(\d+)" % name, out)
+            assert use, name
+            assert int(use.group(1)) <= most
