@@ -23,7 +23,7 @@
 #include "adc_table_tc.h"
 #include "bang_internal.h"
 #include "rerank.h"
-#include "search_kernel.cuh"
+#include "search_team.cuh"
 
 namespace {
 
@@ -557,6 +557,7 @@ void set_graph_args(const bang_index *ix, bang::SearchArgs &a)
         a.adj_stride = ix->rec_words;
         a.base = rec + ix->rec_row_words;
         a.vstride = ix->rec_words * 4u / (uint32_t)elem_size(ix->dtype);
+        a.base_link = 1u;
         return;
     }
     if (ix->placement & BANG_GRAPH_IN_HBM) a.adj = static_cast<const uint32_t *>(ix->adj_hbm.p);
@@ -564,6 +565,7 @@ void set_graph_args(const bang_index *ix, bang::SearchArgs &a)
     a.adj_stride = a.adj_row_words;
     a.base = (ix->placement & BANG_VECTORS_IN_HBM) ? ix->base_hbm.p : ix->base.dev;
     a.vstride = ix->d;
+    a.base_link = (ix->placement & BANG_VECTORS_IN_HBM) ? 0u : 1u;
 }
 
 }  // namespace
@@ -940,6 +942,25 @@ int bang::search_batched(bang_index *ix, const void *queries, uint32_t nq, const
 }
 
 extern "C" {
+
+int bang_internal_form(int dtype, uint64_t n, uint32_t d, uint32_t M, uint32_t R, uint32_t mode, uint32_t log2z,
+                       uint32_t L, uint32_t k, uint32_t nq, uint32_t link, uint32_t batched, uint32_t overlapped,
+                       uint32_t sms, uint32_t *bytes)
+{
+    static unsigned int counter;
+    bang::SearchArgs a;
+    std::memset(&a, 0, sizeof a);
+    a.n = static_cast<uint32_t>(n); a.d = d; a.M = M; a.Mpad = (M + 15u) & ~15u; a.R = R;
+    a.log2z = log2z; a.L = L; a.k = k; a.nq = nq;
+    a.vecb_ok = d % 4 == 0 ? 1u : 0u;
+    a.base_link = link;
+    a.overlapped = overlapped;
+    if (batched) a.queue = &counter;
+    const uint32_t one = bang::SmemLayout(M, log2z, L, k, d, R, static_cast<int>(mode)).total;
+    const uint32_t e = bang::team_expanders(a, dtype, static_cast<int>(mode), sms, one);
+    if (bytes) *bytes = e ? bang::TeamLayout(M, log2z, L, k, d, R, static_cast<int>(mode), e).total : one;
+    return static_cast<int>(1u + e);
+}
 
 int bang_internal_search(bang_index *ix, const void *queries, uint32_t nq, const uint32_t *k_per_q,
                          const uint32_t *L_per_q, uint32_t k, uint32_t L, const bang_search_params *params,

@@ -44,6 +44,12 @@ int bang_internal_search(bang_index *ix, const void *queries, uint32_t nq, const
                          const uint32_t *L_per_q, uint32_t k, uint32_t L, const bang_search_params *params,
                          uint32_t *out_ids, float *out_dist, void *stream, uint32_t form, long long wait_cycles,
                          uint32_t mute, uint32_t *form_out);
+// The form (counted as SearchArgs::form) that a search of such an index with
+// aligned rows takes on a GPU of `sms` SMs, and its shared memory per query.
+// link: vectors read over the host link.  Needs no GPU.
+int bang_internal_form(int dtype, uint64_t n, uint32_t d, uint32_t M, uint32_t R, uint32_t mode, uint32_t log2z,
+                       uint32_t L, uint32_t k, uint32_t nq, uint32_t link, uint32_t batched, uint32_t overlapped,
+                       uint32_t sms, uint32_t *bytes);
 // The launches of a server after this call; no request may be pending or running.
 int bang_internal_server_form(struct bang_server *s, uint32_t form, long long wait_cycles, uint32_t mute);
 int bang_internal_build_shard_graph(int device, const void *base, int dtype, uint64_t n, uint32_t d,

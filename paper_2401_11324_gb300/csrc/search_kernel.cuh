@@ -110,6 +110,7 @@ struct SearchArgs {
     uint32_t *cand_n;
     uint32_t cand_list;       // 1: the candidates are the final worklist instead (cand_cap >= L)
     uint32_t carveout;        // preferred shared-memory share of L1 in percent (0: the CUDA driver's choice)
+    uint32_t base_link;       // `base` is read over the host link (chooses the form of the search only)
     uint32_t overlapped;      // other launches share the GPU (chooses the form of the search only)
     uint32_t form;            // 0: chosen at the launch; 1: one warp a query; 1 + E: a team with E expanders
     uint32_t *form_out;       // host memory or null: the form launched, counted like `form`

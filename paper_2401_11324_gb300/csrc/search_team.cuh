@@ -848,40 +848,117 @@ __global__ void __maxnreg__(team_regs(DCH, MODE)) team_kernel(const SearchArgs a
     }
 }
 
-// Expanders per query, 0 for the one-warp form.  What counts is how many
-// queries share an SM: c of them, limited by their shared memory or by their
-// number.  The team form fills an SM that holds few (the FP32 table's five,
-// the BF16 table's eight, or a small batch); where many one-warp queries fit,
-// they hide one another's latency with fewer instructions.  Measured (GB300,
-// us per call, 200,000 points, L = 100, k = 10, one warp -> 1 / 2 / 3 expanders):
-//   u8 FP32   nq 10,000 (c =  5)  3,292 -> 3,132 / 2,844 / 2,573
-//   u8 BF16   nq 10,000 (c =  8)  2,332 -> 2,416 / 2,273 / 2,438
-//   int8 BF16 nq  6,000 (c =  6)  2,195 -> 2,117 / 1,738 / 1,598
-//   u8 8-bit  nq 10,000 (c = 15)  1,694 -> 2,055 / 2,527 / 3,101
-//   u8 8-bit  nq    600 (c =  4)    405 ->   367 /   350 /   347
-//   u8 exact  nq 10,000 (c = 20)  1,313 -> 1,515 / 1,738 / 1,853
-//   u8 exact  nq      1 (c =  1)    227 ->   196 /   164 /   147
-// hence about 27 warps an SM, at most three expanders (a fourth changed
-// nothing: the control warp is then the slower side), and one warp per query
-// where fewer than two fit.
-inline uint32_t team_expanders(const SearchArgs &a, int mode, int sms)
+// ---- Which form: expanders per query, 0 for one warp.
+//
+// A team answers a query sooner (1.1 to 2.1 times, measured) and takes three or
+// four times the warps.  What counts is how many queries an SM holds at once in
+// either form, by shared memory and registers, and how often it has to be
+// filled for all of them (waves).  Where the team costs no resident query it is
+// the faster form nearly everywhere; where it costs some, its gain has to make
+// up for the waves it adds.  Where it does is read off 4,900 measured points:
+// ten shapes (uint8, int8, FP32; d = 96 to 200, M = 30 to 74, 32 to 68
+// neighbours), all modes, filters of 2^14 to 2^17 bits, L = 32 to 256, 1 to
+// 10,000 queries, graph and vectors in HBM or host memory, plain and batched,
+// indexes inside the L2 cache (60,000 and 100,000 points) and beyond it
+// (700,000).  29 points are more than 2 % slower than one warp, by 11 % at most
+// (by shared memory alone, as it was before: 326, by up to 45 %).  For example,
+// us per call with one warp / two / three expanders, [chosen]; queries that an
+// SM holds in brackets:
+//   u8 d = 128, M = 32  FP32  L = 150     1 query   (5 5 5)   296 /   241 / [200]
+//   the same                          1,200 queries (5 5 5)   652 /   556 / [481]
+//   the same, 8-bit, 2^17             1,200         (8 7 6)  [405]/   596 /  609
+//   int8 M = 50, 8-bit, 2^16          1,400         (9 8 6)   800 /  [617]/  566
+//   u8 d = 130, exact                 1,200        (20 5 4) [1,028]/ 1,542 / 1,279
+//   FP32 d = 128, exact, host, L = 64   600        (21 8 6) [5,652]/ 5,620 / 5,815
+// (u8 and int8 rows of 16-byte multiples, exact: measured again with the
+// registers that search_kernel has now, 60,000 and 300,000 points.)
+// At most three expanders: a fourth changed nothing, the control warp is then
+// the slower side.
+
+// Queries that share an SM: with `bytes` of shared memory each, and teams of E
+// expanders with `regs` registers a thread (16,384 in each quarter of the SM).
+inline uint32_t fit_smem(uint32_t bytes)
 {
-    const uint32_t smem = ((TeamLayout(a.M, a.log2z, a.L, a.k, a.d, a.R, mode, 2).total + 127u) & ~127u) + 1024u;
-    const uint32_t fit = 228u * 1024u / smem, share = (a.nq + static_cast<uint32_t>(sms) - 1u) / static_cast<uint32_t>(sms);
-    if (fit == 0u) return 0u;      // two slots are more shared memory than a CTA may have: the one-warp form's fits
-    // launches that overlap (the server's) fill the SMs together, and all take
-    // the same form: 24 requests, BF16 table, L up to 256 (c = 7), against one
-    // warp per query: two expanders 1.02 times as fast, three 1.06; the form
-    // chosen launch by launch, so that both kinds share the SMs, 0.92
-    const uint32_t c = a.overlapped || fit < share ? fit : share;
-    uint32_t e = c > 0 ? 27u / c - (c <= 27u ? 1u : 0u) : 0u;
-    if (a.overlapped) e = c <= 7u ? 3u : 0u;
-    e = e < kTeamMaxExpanders ? e : kTeamMaxExpanders;
-    if (e == 3u) {       // the third slot must not cost a resident query
-        const uint32_t t3 = ((TeamLayout(a.M, a.log2z, a.L, a.k, a.d, a.R, mode, 3).total + 127u) & ~127u) + 1024u;
-        if (228u * 1024u / t3 < c) e = 2u;
+    return bytes > 227u * 1024u ? 0u : 228u * 1024u / (((bytes + 127u) & ~127u) + 1024u);
+}
+inline uint32_t team_fit(const SearchArgs &a, int mode, uint32_t E)
+{
+    const uint32_t regs = static_cast<uint32_t>(team_regs(a.d > 128u ? 4 : 1, mode));
+    const uint32_t s = fit_smem(TeamLayout(a.M, a.log2z, a.L, a.k, a.d, a.R, mode, E).total);
+    const uint32_t r = 16384u / (32u * regs) * 4u / (1u + E);
+    return s < r ? s : r;
+}
+
+// f1, f2, f3: the queries an SM holds with one warp, two and three expanders.
+inline uint32_t team_choice(const SearchArgs &a, int dtype, int mode, uint32_t sms, uint32_t f1, uint32_t f2,
+                            uint32_t f3)
+{
+    if (a.overlapped) {
+        // launches that fill the SMs together, all in the same form: 24
+        // requests, BF16 table, L up to 256 (8 7 6): two expanders 1.02 times
+        // as fast as one warp, three 1.06; the form chosen launch by launch,
+        // so that both kinds share the SMs, 0.92.  A few small requests, where
+        // most SMs have one query, gain up to twofold.
+        return fit_smem(TeamLayout(a.M, a.log2z, a.L, a.k, a.d, a.R, mode, 2).total) > 7u ? 0u : 3u;
     }
-    return e >= 2u ? e : 0u;
+    const uint32_t share = (a.nq + sms - 1u) / sms, need = share < f1 ? share : f1;
+    const auto waves = [&](uint32_t f) { return f ? (a.nq + sms * f - 1u) / (sms * f) : ~0u; };
+    const uint32_t w1 = waves(f1), w2 = waves(f2), w3 = waves(f3);
+    const bool flt = dtype == 2, wide = a.d > 128u, wide_r = a.R > 64u;
+    const bool lanes = !flt && !wide && a.d % 16u == 0u && a.vecb_ok;    // exact: a lane per row
+    // beyond the L2 cache a hop takes longer, and the team hides it
+    const bool far = static_cast<uint64_t>(a.n) * (4ull * a.R + a.Mpad + a.d * (flt ? 4ull : 1ull)) > (96ull << 20);
+    if (mode == kModeExact) {
+        if (a.base_link && share > 1u) {
+            // every neighbour measured is a row over the host link, which
+            // expansions in vain and neighbours measured twice load
+            if (flt) return f3 >= need && share <= 2u && a.L >= 64u ? 3u : 0u;
+            if (lanes) {
+                if (share <= 2u) return a.L >= 96u && f3 >= need ? 3u : a.L >= 48u && f2 >= need ? 2u : 0u;
+                // rows that fill a 128-byte line: 5 to 10 % better than one
+                // warp's whole-row loads where the search is long
+                if (a.d > 112u && !wide_r && a.L >= 96u) return 2u;
+                return share <= 4u && a.L >= 160u && f2 >= need ? 2u : 0u;
+            }
+        }
+        if (wide && !a.vecb_ok) return f3 >= need && share <= 4u ? 3u : 0u;   // rows read byte by byte
+        if (f3 >= need) return 3u;
+        if (f2 >= need) return 2u;
+        if (a.base_link) return 0u;
+        if (wide) return flt && share <= (a.L >= 128u ? 8u : 6u) ? 3u : 0u;
+        return share <= 9u && (flt || (far && !lanes)) ? 3u : 0u;
+    }
+    // short code rows in the 8-bit table, several waves: one warp has the fewest instructions
+    if (mode == kModeQ8 && a.Mpad <= 32u && a.R > 32u && f1 >= 7u && w1 >= 4u) return 0u;
+    if (f3 >= need) return 3u;
+    const uint32_t e = f3 == f2 || (w3 == w2 && !flt && (wide || (mode == kModeF32 && w2 <= 2u))) ? 3u : 2u;
+    if (f2 >= need) return e;
+    // from here on a team costs resident queries
+    if (mode == kModeF32) {
+        if (w1 > 1u) return e;
+        return !wide && a.Mpad <= 32u && !flt && a.vecb_ok && !wide_r ? 0u : 3u;
+    }
+    if (w1 == 1u) {              // one warp per query holds them all at once
+        if (wide) return flt ? (w2 == 2u ? 2u : 0u) : w3 == 2u && !a.queue ? 3u : 0u;
+        if (f1 <= 7u) return a.Mpad > 32u ? e : 0u;
+        return far && !lanes && !flt && f1 <= 12u ? 2u : 0u;
+    }
+    if (f1 <= 6u) return e;
+    if (wide) return wide_r && f1 > 7u && !flt ? (w1 == 2u && w2 <= 3u ? e : 0u) : f1 <= 9u ? e : 0u;
+    if (f1 == 7u) return !wide_r || w1 <= (far ? 4u : 3u) ? e : 0u;
+    if (f1 > 10u) return 0u;
+    if (wide_r) return w1 == 2u && w2 <= (far ? 3u : 2u) ? 2u : 0u;
+    if (w2 <= w1) return 2u;
+    return a.Mpad >= 64u && f1 <= 9u && ((w1 <= 3u && (far || a.Mpad >= 80u)) || (far && !lanes)) ? 2u : 0u;
+}
+
+// bytes1: the one-warp form's shared memory per query.
+inline uint32_t team_expanders(const SearchArgs &a, int dtype, int mode, uint32_t sms, uint32_t bytes1)
+{
+    const uint32_t f1 = fit_smem(bytes1), f2 = team_fit(a, mode, 2), f3 = team_fit(a, mode, 3);
+    if (f1 == 0u || f2 == 0u) return 0u;
+    const uint32_t e = team_choice(a, dtype, mode, sms, f1 < 32u ? f1 : 32u, f2, f3);
+    return e == 3u && f3 == 0u ? 2u : e;          // three slots may not fit where two do
 }
 
 template <int DT, int RPL, int DCH, int MODE>
@@ -923,7 +1000,7 @@ template <int MODE> cudaError_t launch_team(const SearchArgs &args, int dtype, s
     if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
     if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
     const bool one = a.phase_cycles || a.ncodes;
-    const uint32_t nexp = a.form ? a.form - 1u : one ? 0u : team_expanders(a, MODE, sms);
+    const uint32_t nexp = a.form ? a.form - 1u : one ? 0u : team_expanders(a, dtype, MODE, static_cast<uint32_t>(sms), static_cast<uint32_t>(smem));
     if (a.form > 1u && (one || nexp > kTeamMaxExpanders ||
                         TeamLayout(a.M, a.log2z, a.L, a.k, a.d, a.R, MODE, nexp).total > 227u * 1024u))
         return cudaErrorInvalidValue;            // asked for by name, but not possible here

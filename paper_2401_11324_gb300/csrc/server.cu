@@ -331,7 +331,8 @@ int bang_server_start(bang_index *ix, const bang_server_config *cfg, bang_server
             release_all(s.get());
             return sfail(BANG_ECUDA, "bang_server_start: stream creation failed");
         }
-        // one empty launch per stream allocates its work counter up front
+        // one empty launch per stream allocates its work counter up front and
+        // loads the kernel that its launches run
         const Views dv = views(s->d_arena, s.get(), 1);
         const uint32_t one = 1, kL = cfg->k_max;
         cudaMemsetAsync(dv.q, 0, d * s->esz, st.stream);
@@ -342,8 +343,8 @@ int bang_server_start(bang_index *ix, const bang_server_config *cfg, bang_server
         p.mode = cfg->mode;
         p.bloom_log2 = cfg->bloom_log2;
         p.early_codes = cfg->early_codes;
-        int rc = bang_search_batched(ix, dv.q, 1, dv.k, dv.L, cfg->k_max, cfg->L_max, &p, dv.ids, dv.dist,
-                                     st.stream);
+        int rc = bang::search_batched(ix, dv.q, 1, dv.k, dv.L, cfg->k_max, cfg->L_max, &p, dv.ids, dv.dist,
+                                      st.stream, s->form);
         if (rc != BANG_OK || cudaStreamSynchronize(st.stream) != cudaSuccess) {
             std::string m = std::string("bang_server_start: warm-up search failed: ") + bang_last_error();
             release_all(s.get());

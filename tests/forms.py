@@ -43,3 +43,11 @@ def shard_graph(X, centres, ell, R, Lb, alpha, batch_frac, log2z, form=0, wait_c
                   Lb, alpha, batch_frac, log2z, 0, bang._ptr(adj), None, None, form, wait_cycles,
                   0 if mute is None else 1 + mute))
     return adj
+
+
+def choice(dtype, n, d, M, R, mode, log2z, L, k, nq, link=0, batched=0, overlapped=0, sms=152):
+    """(form, shared memory per query) that the library takes; needs no GPU."""
+    b = ctypes.c_uint32(0)
+    f = bang.lib().bang_internal_form
+    f.argtypes = [ctypes.c_int, ctypes.c_uint64] + [ctypes.c_uint32] * 12 + [ctypes.c_void_p]
+    return f(dtype, n, d, M, R, mode, log2z, L, k, nq, link, batched, overlapped, sms, ctypes.addressof(b)), b.value
