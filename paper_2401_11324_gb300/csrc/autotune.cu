@@ -42,6 +42,7 @@ struct Runner {
     float *d_dist = nullptr;
     cudaEvent_t e0 = nullptr, e1 = nullptr;
     std::vector<uint32_t> ids;
+    uint32_t form = 0;          // of the last run: 1 one warp per query, else a team
 
     int init(uint32_t L_max)
     {
@@ -83,12 +84,13 @@ struct Runner {
         p.prefetch_depth = c.depth;
         p.early_codes = c.early;
         p.rerank = c.rerank;
-        if (!batched) return bang_search(ix, queries, nq, k, c.L, &p, d_ids, d_dist, st);
+        if (!batched)
+            return bang_internal_search(ix, queries, nq, nullptr, nullptr, k, c.L, &p, d_ids, d_dist, st, 0, 0, 0, &form);
         std::vector<uint32_t> Lq(nq, c.L);
         if (cudaMemcpyAsync(d_Lq, Lq.data(), sizeof(uint32_t) * nq, cudaMemcpyHostToDevice, st) != cudaSuccess ||
             cudaStreamSynchronize(st) != cudaSuccess)
             return BANG_ECUDA;
-        return bang_search_batched(ix, queries, nq, d_kq, d_Lq, k, c.L, &p, d_ids, d_dist, st);
+        return bang_internal_search(ix, queries, nq, d_kq, d_Lq, k, c.L, &p, d_ids, d_dist, st, 0, 0, 0, &form);
     }
     // Mean milliseconds per batch over `reps` launches after one warm-up.
     int time(const Cfg &c, uint32_t reps, float *ms)
@@ -408,7 +410,9 @@ extern "C" int bang_autotune(bang_index *ix, const void *queries, uint32_t nq, u
             return rc;
         }
     }
-    if (o.try_prefetch_depth) {       // the winner with the speculative request too (same results)
+    if ((o.try_prefetch_depth || o.try_structure) && (rc = run.run(best_c))) return rc;
+    const bool alone = run.form == 1u;        // a team of warps ignores both kinds of requests ahead
+    if (o.try_prefetch_depth && alone) {      // the winner with the speculative request too (same results)
         Cfg c2 = best_c;
         c2.depth = 2;
         float ms2 = 0.f;
@@ -423,15 +427,17 @@ extern "C" int bang_autotune(bang_index *ix, const void *queries, uint32_t nq, u
     if (o.try_structure && best_c.mode != BANG_MODE_EXACT) {
         // the winner with early code rows, then with the re-rank staged
         // (same results: each kept only if faster)
-        Cfg c3 = best_c;
-        c3.early = 1;
-        float ms3 = 0.f;
-        if ((rc = run.time(c3, o.reps, &ms3))) return rc;
-        ++out->candidates;
-        if (ms3 < out->ms) {
-            out->ms = ms3;
-            out->early_codes = 1;
-            best_c = c3;
+        if (alone) {
+            Cfg c3 = best_c;
+            c3.early = 1;
+            float ms3 = 0.f;
+            if ((rc = run.time(c3, o.reps, &ms3))) return rc;
+            ++out->candidates;
+            if (ms3 < out->ms) {
+                out->ms = ms3;
+                out->early_codes = 1;
+                best_c = c3;
+            }
         }
         Cfg c4 = best_c;
         c4.rerank = 1;

@@ -132,3 +132,20 @@ def test_structure_timed_on_the_winner(setup, tmp_path):
     assert r2["from_cache"] == 1
     for f in ("mode", "bloom_log2", "L", "early_codes", "rerank"):
         assert r2[f] == r[f], f
+
+
+def test_requests_ahead_are_not_tuned_where_a_team_searches(setup):
+    # with the FP32 table a team of warps searches each of these queries, which
+    # has neither early code rows nor a speculative request: neither is timed
+    # nor chosen.  One warp per query (large batches on the 8-bit table) has both
+    w, ix, q = setup
+    truth = np.ascontiguousarray(w["gt_ids"][:, :10])
+    kw = dict(bloom_min=16, bloom_max=16, try_tensor_tables=0, try_prefetch_depth=1, try_structure=1)
+    for _ in range(5):
+        r = ix.autotune(q, 10, 64, truth=truth, modes=1 << 0, **kw)
+        assert r["prefetch_depth"] == 1 and r["early_codes"] == 0
+        assert r["candidates"] == 2                  # the form and its staged re-rank
+    many = q.repeat(-(-5000 // q.shape[0]), 1).contiguous()
+    many_truth = np.tile(truth, (many.shape[0] // q.shape[0], 1))
+    r = ix.autotune(many, 10, 64, truth=many_truth, modes=1 << 3, **kw)
+    assert r["candidates"] == 4
