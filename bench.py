@@ -440,8 +440,9 @@ def large_workload(args, device):
 # log2, what).  Results do not depend on the placement (tested), so every
 # operating point is found with graph and vectors in HBM.
 # early: request every neighbour's code row as soon as the node's row arrives
-# (early_codes; same results; measured faster with the FP32 and BF16 tables,
-# slower with the 8-bit table).
+# (early_codes; same results; in the one-warp form of the search measured faster
+# with the FP32 and BF16 tables, slower with the 8-bit table; a team of warps,
+# which searches these forms' batches on the FP32 table, ignores it).
 def _form(name, mode, placement, lz, early, tsrc, what, rerank=0):
     return dict(name=name, mode=mode, placement=placement, lz=lz, early=early, tsrc=tsrc,
                 rerank=rerank, what=what)
@@ -825,10 +826,11 @@ def run_large(args):
         "roofline": {"bound": "hbm", "achieved": hbm_gbs, "peak": hbm_peak, "unit": "GB/s",
                      "frac": hbm_gbs / hbm_peak, "traffic": None,
                      "traffic_note": "not captured at this size (83 GB in HBM); at 8M points "
-                                     "and L = 224 the staged headline's search read 1.917 GB and "
-                                     "its re-rank 0.303 GB of DRAM per step for 1.543 GB "
+                                     "and L = 224 one warp per query read 1.917 GB in the staged "
+                                     "search and 0.303 GB in its re-rank per step for 1.543 GB "
                                      "algorithmic (1.44x: each 32-byte code row costs a 64-byte "
-                                     "DRAM access); the fused form's search read 2.305 GB",
+                                     "DRAM access), 2.305 GB in the fused search; not captured "
+                                     "for the team of warps that runs the headline",
                      "peak_source": "measured (MEASURED_PEAKS.json)" if "hbm_gbs" in peaks
                                     else "fallback",
                      "algorithmic_bytes_per_launch": hbm_bytes,

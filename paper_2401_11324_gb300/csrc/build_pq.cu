@@ -14,7 +14,7 @@
 // a thread, and FP64 runs at a sixtieth of the FP32 rate here.  So every
 // distance is computed in FP32 first, keeping the smallest and the second
 // smallest; the FP64 distances are computed only where the second lies within
-// both values' rounding errors of the smallest (kSlack), and then only for the
+// both values' rounding errors of the smallest (`cut`), and then only for the
 // centroids that do.  The result is the FP64 one always.
 // Update: integer sums are exact in any order, so uint8 and int8 points are
 // added with shared-memory atomics, a block per part of the sample; float

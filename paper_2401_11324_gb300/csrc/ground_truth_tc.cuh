@@ -21,11 +21,13 @@
 // one accumulator while the other is being computed.  Few pairs pass: they are
 // kept in shared memory, 4 per thread, and appended to the query's list with
 // one atomic, by all lanes of a warp together (so the first level, where a tenth
-// of the pairs passes, took 0.64 ms instead of 0.87).  The filter's instructions
-// set the pace (216 per 32 x 32 pairs; 10^10 pairs take the MMAs alone 1.4 ms):
-// with four warps a group, two a scheduler, the three levels of 10,000 queries
-// over 1M points took 7.5 ms (tensor pipe 23 %), with eight 6.1; packed FP32
-// arithmetic with a three-way minimum and loads one step ahead changed nothing.
+// of the pairs passes, took 0.64 ms instead of 0.87).  The filter
+// sets the pace (216 instructions per 32 x 32 pairs; 10^10 pairs take the MMAs
+// alone 1.4 ms): with four warps a group, two a scheduler, the three levels of
+// 10,000 queries over 1M points took 7.5 ms (tensor pipe 23 %), with eight 6.1
+// (27 %; half the issue rate, the warps waiting for the accumulators most);
+// packed FP32 arithmetic with a three-way minimum and loads one step ahead
+// changed nothing.
 #pragma once
 
 #include <cuda_bf16.h>

@@ -955,7 +955,7 @@ __global__ void __launch_bounds__(32, least_queries(DT, RPL, DCH, MODE, PH)) sea
                 // one new neighbour (its whole row) and all of them are
                 // requested at once; the query's words come from shared
                 // memory, 16 bytes at a time to all lanes (10,000 u8 queries
-                // at L = 48: 0.75 ms; as shuffles, one a word, and with the
+                // at L = 48: 0.70 ms; as shuffles, one a word, and with the
                 // keys passed through shared memory, 0.82)
                 in_regs = true;
                 const uint32_t nv = d / 16u;     // 16-byte chunks per row, <= 8
